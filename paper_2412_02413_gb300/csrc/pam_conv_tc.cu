@@ -1,7 +1,9 @@
-// pam_conv_tc.cu -- tensor-core (tcgen05) forward of the 3x3 convolutions of
-// the learned NCC-weight network, for rows of nx = 128 pixels: the first layer
+// pam_conv_tc.cu -- tensor-core (tcgen05) 3x3 convolutions of the learned
+// NCC-weight network, for rows of nx = 128 pixels. Forward: the first layer
 // (5 -> 32, bias, ReLU), the hidden layers (32 -> 32, bias, ReLU) and the last
-// layer (32 -> 1, bias, FP32 output).
+// layer (32 -> 1, bias, FP32 output). Input gradients: the same convolution of
+// dY with the adjoint weights (1 -> 32 or 32 -> 32), zero where the layer's
+// input activation, a ReLU output, is zero.
 //
 // One output row is a GEMM with M = 128 pixels, N = 32 output channels (16
 // for the last layer, whose channels 1..15 carry zero weights) and K = 9 taps
@@ -63,10 +65,63 @@ __device__ __forceinline__ unsigned pack2(float a, float b)
     return r;
 }
 
-template <int NCI, int NCO, bool F32OUT>
+// What the epilogue does with a row: bias and ReLU, bias and FP32 output, or
+// the ReLU mask of an input gradient.
+enum { TC_RELU = 0, TC_F32 = 1, TC_MASK = 2 };
+
+// Each of two packed BF16 values where its mask (a ReLU output: zero or
+// positive) is positive, else zero.
+__device__ __forceinline__ unsigned masked2(unsigned v, unsigned m)
+{
+    const unsigned lo = (m & 0xFFFFu) != 0u && (m & 0x8000u) == 0u ? 0xFFFFu : 0u;
+    const unsigned hi = (m >> 16) != 0u && (m & 0x80000000u) == 0u ? 0xFFFF0000u : 0u;
+    return v & (lo | hi);
+}
+
+// One output in the CUDA-core kernels' order (pam_learn.cu, conv_cc_kernel): a
+// chain of FP32 FMAs over the input channels and, within one, the nine taps.
+// `in` points at the output's pixel in the first of its three padded input rows
+// (chunk planes `plane` apart), `w` at the output channel's weights in the
+// staged [tap][KCH][NCO][8].
+template <int NCI, int KCH, int NCO>
+__device__ float conv_chain(const uint4 *__restrict__ in, size_t plane, const uint8_t *w)
+{
+    float s = 0.0f;
+#pragma unroll 1
+    for (int c = 0; c < NCI; ++c) {
+        uint4 x[9], q[9];
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+            x[t] = in[(size_t)c * plane + (size_t)(t / 3) * WP + t % 3];
+            q[t] = *reinterpret_cast<const uint4 *>(w + (size_t)((t * KCH + c) * NCO) * 16);
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+#pragma unroll
+            for (int t = 0; t < 9; ++t) {
+                const unsigned xw = k < 2 ? x[t].x : k < 4 ? x[t].y : k < 6 ? x[t].z : x[t].w;
+                const unsigned qw = k < 2 ? q[t].x : k < 4 ? q[t].y : k < 6 ? q[t].z : q[t].w;
+                s = fmaf(__uint_as_float((k & 1) ? xw & 0xFFFF0000u : xw << 16),
+                         __uint_as_float((k & 1) ? qw & 0xFFFF0000u : qw << 16), s);
+            }
+    }
+    return s;
+}
+
+// EXACT (training): the outputs are bit for bit those of the CUDA-core kernel,
+// so a gradient does not depend on which of the two computed the activations.
+// Both sum in FP32 and differ by the order only, which shows where a sum lies
+// within that difference of a BF16 rounding boundary or of the ReLU's zero:
+// those outputs (about one in a thousand) are recomputed by conv_chain. The
+// window is CHAIN_TOL times the pixel's largest sum: the chain of up to 288
+// roundings and the tensor core's 18 steps differ by about 1.5e-7 of it (one
+// standard deviation), a sixth of the window.
+constexpr float CHAIN_TOL = 9.5367431640625e-7f;   // 2^-20
+
+template <int NCI, int NCO, int EPI, bool EXACT>
 __global__ void __launch_bounds__(THREADS)
 conv_tc_kernel(const uint4 *__restrict__ in, const uint4 *__restrict__ wt, const float *__restrict__ bias,
-               void *__restrict__ out, int H, int *__restrict__ status)
+               const uint4 *__restrict__ mask, void *__restrict__ out, int H, int *__restrict__ status)
 {
     using CS = ConvShape<NCI, NCO>;
     constexpr int KCH = CS::KCH, ROW_BYTES = CS::ROW_BYTES, WT_BYTES = CS::WT_BYTES;
@@ -200,19 +255,26 @@ conv_tc_kernel(const uint4 *__restrict__ in, const uint4 *__restrict__ wt, const
         }
         __syncwarp();
     } else {
-        // ---------------- epilogue: TMEM -> bias + ReLU -> BF16 ----------------
+        // ---------------- epilogue: TMEM -> bias + ReLU, or the mask -> BF16 ----------------
         const int quarter = warp & 3;
         const int j = 32 * quarter + lane;   // pixel = TMEM lane
-        constexpr int NB = F32OUT ? 1 : 32;
-        float b[NB];
+        constexpr int NB = EPI == TC_F32 ? 1 : EPI == TC_RELU ? 32 : 0;
+        float b[NB ? NB : 1];
 #pragma unroll
         for (int o = 0; o < NB; ++o) b[o] = bias[o];
         for (int r = 0; r < nr; ++r) {
             const int t = r & 1;
+            // the row's mask is read while its MMAs run
+            const size_t at = ((size_t)f * 4 * HP + r_first + r + 1) * WP + (j + 1);
+            uint4 mk[4];
+            if constexpr (EPI == TC_MASK) {
+#pragma unroll
+                for (int ch = 0; ch < 4; ++ch) mk[ch] = mask[at + (size_t)ch * HP * WP];
+            }
             if (!__all_sync(0xffffffffu, wait(&afull[t], (unsigned)(r >> 1) & 1u))) break;
             tc_fence_after();
             const unsigned taddr = tmem + (unsigned)(t * 32) + ((unsigned)(32 * quarter) << 16);
-            if constexpr (F32OUT) {
+            if constexpr (EPI == TC_F32) {
                 unsigned a0;
                 asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n" : "=r"(a0) : "r"(taddr));
                 asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
@@ -227,15 +289,61 @@ conv_tc_kernel(const uint4 *__restrict__ in, const uint4 *__restrict__ wt, const
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&aempty[t]);
-                const int prow = r_first + r + 1;
-                uint4 *dst = reinterpret_cast<uint4 *>(out) + (((size_t)f * 4) * HP + prow) * WP + (j + 1);
+                uint4 *dst = reinterpret_cast<uint4 *>(out) + at;
+                unsigned redo = 0u;   // bit o: output o is too near a boundary
+                if constexpr (EXACT) {
+                    float top = 0.0f;
+#pragma unroll
+                    for (int o = 0; o < 32; ++o) top = fmaxf(top, fabsf(__uint_as_float(acc[o])));
+                    const float tol = CHAIN_TOL * top;
+#pragma unroll
+                    for (int o = 0; o < 32; ++o) {
+                        float v = __uint_as_float(acc[o]);
+                        if constexpr (EPI == TC_RELU) v += b[o];
+                        float up = v + tol, dn = v - tol;
+                        if constexpr (EPI == TC_RELU) {
+                            up = fmaxf(up, 0.0f);
+                            dn = fmaxf(dn, 0.0f);
+                        }
+                        const unsigned pk = pack2(up, dn);
+                        if ((pk >> 16) != (pk & 0xFFFFu)) redo |= 1u << o;
+                    }
+                }
 #pragma unroll
                 for (int ch = 0; ch < 4; ++ch) {
                     float y[8];
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) y[k] = fmaxf(__uint_as_float(acc[ch * 8 + k]) + b[ch * 8 + k], 0.0f);
-                    dst[(size_t)ch * HP * WP] =
-                        make_uint4(pack2(y[0], y[1]), pack2(y[2], y[3]), pack2(y[4], y[5]), pack2(y[6], y[7]));
+                    for (int k = 0; k < 8; ++k) {
+                        y[k] = __uint_as_float(acc[ch * 8 + k]);
+                        if constexpr (EPI == TC_RELU) y[k] = fmaxf(y[k] + b[ch * 8 + k], 0.0f);
+                    }
+                    uint4 v = make_uint4(pack2(y[0], y[1]), pack2(y[2], y[3]), pack2(y[4], y[5]), pack2(y[6], y[7]));
+                    if constexpr (EPI == TC_MASK)
+                        v = make_uint4(masked2(v.x, mk[ch].x), masked2(v.y, mk[ch].y), masked2(v.z, mk[ch].z),
+                                       masked2(v.w, mk[ch].w));
+                    dst[(size_t)ch * HP * WP] = v;
+                }
+                if constexpr (EXACT) {
+                    // each lane patches its own pixel's outputs, one per turn of the warp's loop
+                    const uint4 *src = in + ((size_t)f * NCI * HP + r_first + r) * WP + j;
+                    while (__any_sync(0xffffffffu, redo != 0u)) {
+                        if (redo != 0u) {
+                            const int o = __ffs(redo) - 1;
+                            redo &= redo - 1u;
+                            float v = conv_chain<NCI, KCH, NCO>(src, (size_t)HP * WP, sW + (size_t)o * 16);
+                            if constexpr (EPI == TC_RELU) v = fmaxf(v + bias[o], 0.0f);
+                            bool live = true;
+                            if constexpr (EPI == TC_MASK) {
+                                const unsigned short m = reinterpret_cast<const unsigned short *>(
+                                    mask + at + (size_t)(o >> 3) * HP * WP)[o & 7];
+                                live = m != 0u && (m & 0x8000u) == 0u;
+                            }
+                            if (live)
+                                reinterpret_cast<unsigned short *>(dst + (size_t)(o >> 3) * HP * WP)[o & 7] =
+                                    (unsigned short)(pack2(v, v) & 0xFFFFu);
+                        }
+                        __syncwarp();
+                    }
                 }
             }
         }
@@ -247,19 +355,20 @@ conv_tc_kernel(const uint4 *__restrict__ in, const uint4 *__restrict__ wt, const
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(64u) : "memory");
 }
 
-template <int NCI, int NCO, bool F32OUT>
+template <int NCI, int NCO, int EPI, bool EXACT>
 cudaError_t set_tc_smem()
 {
-    return cudaFuncSetAttribute(conv_tc_kernel<NCI, NCO, F32OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(conv_tc_kernel<NCI, NCO, EPI, EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)ConvShape<NCI, NCO>::SMEM);
 }
 
-template <int NCI, int NCO, bool F32OUT>
-cudaError_t launch_tc(const uint4 *in, const uint4 *wt, const float *bias, void *out, int F, int H, int *status,
-                      cudaStream_t st)
+template <int NCI, int NCO, int EPI, bool EXACT>
+cudaError_t launch_tc(const uint4 *in, const uint4 *wt, const float *bias, const uint4 *mask, void *out, int F, int H,
+                      int *status, cudaStream_t st)
 {
     dim3 grid((H + ROWS - 1) / ROWS, F);
-    conv_tc_kernel<NCI, NCO, F32OUT><<<grid, THREADS, ConvShape<NCI, NCO>::SMEM, st>>>(in, wt, bias, out, H, status);
+    conv_tc_kernel<NCI, NCO, EPI, EXACT><<<grid, THREADS, ConvShape<NCI, NCO>::SMEM, st>>>(in, wt, bias, mask, out, H,
+                                                                                           status);
     return cudaGetLastError();
 }
 
@@ -267,18 +376,36 @@ cudaError_t launch_tc(const uint4 *in, const uint4 *wt, const float *bias, void 
 
 cudaError_t prepare_conv_tc()
 {
-    cudaError_t e = set_tc_smem<1, 32, false>();
-    if (e == cudaSuccess) e = set_tc_smem<4, 32, false>();
-    if (e == cudaSuccess) e = set_tc_smem<4, 16, true>();
+    cudaError_t e = set_tc_smem<1, 32, TC_RELU, false>();
+    if (e == cudaSuccess) e = set_tc_smem<4, 32, TC_RELU, false>();
+    if (e == cudaSuccess) e = set_tc_smem<4, 16, TC_F32, false>();
+    if (e == cudaSuccess) e = set_tc_smem<1, 32, TC_RELU, true>();
+    if (e == cudaSuccess) e = set_tc_smem<4, 32, TC_RELU, true>();
+    if (e == cudaSuccess) e = set_tc_smem<1, 32, TC_MASK, true>();
+    if (e == cudaSuccess) e = set_tc_smem<4, 32, TC_MASK, true>();
     return e;
 }
 
 cudaError_t launch_conv_tc(int layer, const uint4 *in, const uint4 *wt, const float *bias, void *out, int F, int H,
                            int *status, cudaStream_t st)
 {
-    if (layer == 0) return launch_tc<1, 32, false>(in, wt, bias, out, F, H, status, st);
-    if (layer == 4) return launch_tc<4, 16, true>(in, wt, bias, out, F, H, status, st);
-    return launch_tc<4, 32, false>(in, wt, bias, out, F, H, status, st);
+    if (layer == 0) return launch_tc<1, 32, TC_RELU, false>(in, wt, bias, nullptr, out, F, H, status, st);
+    if (layer == 4) return launch_tc<4, 16, TC_F32, false>(in, wt, bias, nullptr, out, F, H, status, st);
+    return launch_tc<4, 32, TC_RELU, false>(in, wt, bias, nullptr, out, F, H, status, st);
+}
+
+cudaError_t launch_conv_tc_exact(int layer, const uint4 *in, const uint4 *wt, const float *bias, uint4 *out, int F,
+                                 int H, int *status, cudaStream_t st)
+{
+    if (layer == 0) return launch_tc<1, 32, TC_RELU, true>(in, wt, bias, nullptr, out, F, H, status, st);
+    return launch_tc<4, 32, TC_RELU, true>(in, wt, bias, nullptr, out, F, H, status, st);
+}
+
+cudaError_t launch_conv_tc_grad(int layer, const uint4 *dY, const uint4 *wt, const uint4 *mask, uint4 *out, int F,
+                                int H, int *status, cudaStream_t st)
+{
+    if (layer == 4) return launch_tc<1, 32, TC_MASK, true>(dY, wt, nullptr, mask, out, F, H, status, st);
+    return launch_tc<4, 32, TC_MASK, true>(dY, wt, nullptr, mask, out, F, H, status, st);
 }
 
 }  // namespace pam

@@ -15,8 +15,10 @@
 // [F][C/8][nz+2][nx+2][8], eight channels of one pixel in 16 bytes, with a
 // zero border of one pixel so that every 3x3 tap reads memory.
 //
-// Kernels of this file run on CUDA cores; the forward of every layer also has
-// a tcgen05 tensor-core version (pam_conv_tc.cu) for nx = 128.
+// The convolutions of this file run on CUDA cores; the forward and the input
+// gradient of every layer also have a tcgen05 tensor-core version
+// (pam_conv_tc.cu) for nx = 128, and the weight gradients run on the tensor
+// cores at every width (pam_wgrad.cu).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -37,6 +39,20 @@ namespace pam {
 cudaError_t launch_conv_tc(int layer, const uint4 *in, const uint4 *wt, const float *bias, void *out, int F, int H,
                            int *status, cudaStream_t st);
 cudaError_t prepare_conv_tc();
+// Hidden layers 0..3 for training: the same bits as the CUDA-core kernel's.
+cudaError_t launch_conv_tc_exact(int layer, const uint4 *in, const uint4 *wt, const float *bias, uint4 *out, int F,
+                                 int H, int *status, cudaStream_t st);
+// tcgen05 input gradient of layer 1..4 through the ReLU of its input: the
+// convolution of dY with the adjoint weights, zero where `mask` (the layer's
+// input activation) is not positive; nx == 128 only, the CUDA-core kernel's bits.
+cudaError_t launch_conv_tc_grad(int layer, const uint4 *dY, const uint4 *wt, const uint4 *mask, uint4 *out, int F,
+                                int H, int *status, cudaStream_t st);
+// Weight gradients on the tensor cores (pam_wgrad.cu): wgrad_ctas partials of
+// the layer's parameters (w, then b), every width.
+cudaError_t prepare_wgrad();
+int wgrad_ctas(int n_sms, int F, int H);
+cudaError_t launch_wgrad(int layer, const uint4 *X, const uint4 *dY, int F, int H, int W, int ctas, float *part,
+                         int *status, cudaStream_t st);
 
 namespace {
 
@@ -50,13 +66,15 @@ __host__ __device__ constexpr int TC_KCH(int l) { return l == 0 ? 2 : 4; }
 __host__ __device__ constexpr int TC_NCO(int l) { return l == NL - 1 ? 16 : 32; }
 __host__ __device__ constexpr size_t tc_count(int l) { return (size_t)9 * TC_KCH(l) * TC_NCO(l) * 8; }
 __host__ __device__ constexpr size_t tc_offset(int l) { return l == 0 ? 0 : tc_offset(l - 1) + tc_count(l - 1); }
+// tensor-core layout of layer l's adjoint (l >= 1): [9][TCB_KCH][32][8] BF16
+__host__ __device__ constexpr int TCB_KCH(int l) { return l == NL - 1 ? 2 : 4; }
+__host__ __device__ constexpr size_t tcb_count(int l) { return l == 0 ? 0 : (size_t)9 * TCB_KCH(l) * 32 * 8; }
+__host__ __device__ constexpr size_t tcb_offset(int l) { return l == 0 ? tc_offset(NL) : tcb_offset(l - 1) + tcb_count(l - 1); }
 constexpr int N_BANDS = 4;
 constexpr float FEATURE_FLOOR = 1e-4f;
 constexpr float WEIGHT_FLOOR = 0.05f;   // loss weight w = floor + (1 - floor) min(1, E / max E)
 constexpr int CT = 128;        // threads (= pixels along a row) of a CUDA-core conv block
 constexpr int PR = 2;          // output rows per conv block
-constexpr int WSPLIT = 131;    // padded row stride (floats) of the weight-gradient staging; odd: no bank conflicts
-constexpr int RS = 16;         // rows per weight-gradient block
 constexpr int EPI_THREADS = 256;
 
 __host__ __device__ constexpr size_t w_count(int l) { return (size_t)COUT(l) * CIN(l) * 9; }
@@ -87,6 +105,7 @@ struct PrepPtrs {
     float *wb[NL];
     float *bias[NL];
     uint16_t *wtc[NL];
+    uint16_t *wtcb[NL];
 };
 
 __global__ void prep_kernel(const float *__restrict__ params, PrepPtrs pp)
@@ -117,6 +136,13 @@ __global__ void prep_kernel(const float *__restrict__ params, PrepPtrs pp)
             const float v = (o < co && c < ci) ? w[((size_t)o * ci + c) * 9 + t] : 0.0f;
             pp.wtc[l][i] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
         }
+    }
+    // the adjoint in the same layout: [tap][chunk of 8 output channels][input channel][8]
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (int)tcb_count(l); i += gridDim.x * blockDim.x) {
+        const int k = i % 8, c = (i / 8) % 32, ch = (i / 256) % TCB_KCH(l), t = i / (256 * TCB_KCH(l));
+        const int o = ch * 8 + k;
+        const float v = o < co ? w[((size_t)o * ci + c) * 9 + (8 - t)] : 0.0f;
+        pp.wtcb[l][i] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
     }
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < co; i += gridDim.x * blockDim.x) pp.bias[l][i] = b[i];
 }
@@ -309,139 +335,33 @@ conv_cc_kernel(const uint4 *__restrict__ in, const float *__restrict__ wt, const
     }
 }
 
-// -------------------------------------------- convolution (weight grad) ----
-// dW[o][c][u][v] = sum_{n,i,j} dY[n][o][i][j] X[n][c][i+u-1][j+v-1], db[o] = sum dY.
-// Block = RS rows of one frame; per row it stages three input rows (FP32,
-// channel-major, stride WSPLIT) and the row of dY, and each thread accumulates
-// OG output channels x one input channel x 9 taps over its range of pixels with
-// a sliding window along the row. Partial sums per block go to `part`
-// ([block][COUT][CI][9] then [block][COUT] for db) and are summed in block order.
-// Staging (inputs + dY row) or, at the end, the split reduction buffer
-// [PXS][NCOMBO][OG * 10], whichever is larger.
-template <int NCI, int NCO>
-constexpr size_t wgrad_smem()
+// Sum of the weight gradients' partials over the CTAs, in a fixed order, into
+// the gradient vector. Layer l's partials are [n][p_count(l)] from n p_offset(l).
+// Latency-bound (the partials sit in L2): 8 threads of a block share a
+// parameter's partials, so that a thread's chain is n / 8 loads with several in
+// flight. One launch for all layers: 9 us for 152 partials, where one launch
+// per layer with one thread per parameter took 110 us each for 512.
+constexpr int RED_Y = 8;
+__global__ void __launch_bounds__(32 * RED_Y) wgrad_reduce_kernel(const float *__restrict__ part, int n,
+                                                                  float *__restrict__ grads)
 {
-    constexpr size_t stage = (size_t)3 * NCI * 8 * WSPLIT * 4 + (size_t)NCO * (CT + 1) * 4;
-    constexpr size_t red = (size_t)256 * (NCO >= 4 ? 4 : 1) * 10 * 4;
-    return stage > red ? stage : red;
-}
-
-template <int NCI, int NCO>
-__global__ void __launch_bounds__(256)
-wgrad_kernel(const uint4 *__restrict__ X, const uint4 *__restrict__ dY, int H, int W, float *__restrict__ part)
-{
-    constexpr int CI = NCI * 8, OG = NCO >= 4 ? 4 : 1, NOG = NCO / OG, NCOMBO = CI * NOG;
-    constexpr int PXS = 256 / NCOMBO;
-    static_assert(PXS >= 1 && NCOMBO * PXS == 256, "thread mapping of the weight gradient");
-    constexpr int NCY = (NCO + 7) / 8;      // chunks of dY
-    extern __shared__ __align__(16) unsigned char smem[];
-    float *sX = reinterpret_cast<float *>(smem);             // [3][CI][WSPLIT]
-    float *sY = sX + 3 * CI * WSPLIT;                        // [NCO][CT+1]
-    const int tid = threadIdx.x;
-    const int c = tid % CI, og = (tid / CI) % NOG, s = tid / NCOMBO;
-    const int f = blockIdx.y, strip = blockIdx.x;
-    const int HP = H + 2, WP = W + 2;
-    const int p_lo = s * W / PXS, p_hi = (s + 1) * W / PXS;
-
-    float acc[OG][9], db[OG];
-#pragma unroll
-    for (int k = 0; k < OG; ++k) {
-        db[k] = 0.0f;
-#pragma unroll
-        for (int t = 0; t < 9; ++t) acc[k][t] = 0.0f;
+    __shared__ float sh[RED_Y][32];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + tx;
+    float s = 0.0f;
+    if (i < (int)N_PARAMS) {
+        int l = 0;
+        while (l + 1 < NL && i >= (int)p_offset(l + 1)) ++l;
+        const size_t stride = p_count(l);
+        const float *src = part + (size_t)n * p_offset(l) + (i - p_offset(l));
+#pragma unroll 4
+        for (int b = ty; b < n; b += RED_Y) s += src[(size_t)b * stride];
     }
-    for (int i = strip * RS; i < min(H, strip * RS + RS); ++i) {
-        __syncthreads();
-        for (int idx = tid; idx < 3 * NCI * WSPLIT; idx += 256) {
-            const int u = idx / (NCI * WSPLIT), rem = idx % (NCI * WSPLIT), ch = rem / WSPLIT, px = rem % WSPLIT;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (px < WP) v = X[(((size_t)f * NCI + ch) * HP + (i + u)) * WP + px];
-            float *d = sX + ((size_t)u * CI + ch * 8) * WSPLIT + px;
-            d[0] = bf_lo(v.x); d[WSPLIT] = bf_hi(v.x);
-            d[2 * WSPLIT] = bf_lo(v.y); d[3 * WSPLIT] = bf_hi(v.y);
-            d[4 * WSPLIT] = bf_lo(v.z); d[5 * WSPLIT] = bf_hi(v.z);
-            d[6 * WSPLIT] = bf_lo(v.w); d[7 * WSPLIT] = bf_hi(v.w);
-        }
-        for (int idx = tid; idx < NCY * W; idx += 256) {
-            const int ch = idx / W, px = idx % W;
-            const uint4 v = dY[(((size_t)f * NCY + ch) * HP + (i + 1)) * WP + (px + 1)];
-            const float y8[8] = {bf_lo(v.x), bf_hi(v.x), bf_lo(v.y), bf_hi(v.y),
-                                 bf_lo(v.z), bf_hi(v.z), bf_lo(v.w), bf_hi(v.w)};
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if (ch * 8 + k < NCO) sY[(ch * 8 + k) * (CT + 1) + px] = y8[k];
-        }
-        __syncthreads();
-        if (p_lo < p_hi) {
-            float xw[3][3];
-#pragma unroll
-            for (int u = 0; u < 3; ++u)
-#pragma unroll
-                for (int v = 0; v < 2; ++v) xw[u][v + 1] = sX[((size_t)u * CI + c) * WSPLIT + p_lo + v];
-            for (int px = p_lo; px < p_hi; ++px) {
-#pragma unroll
-                for (int u = 0; u < 3; ++u) {
-                    xw[u][0] = xw[u][1];
-                    xw[u][1] = xw[u][2];
-                    xw[u][2] = sX[((size_t)u * CI + c) * WSPLIT + px + 2];
-                }
-#pragma unroll
-                for (int k = 0; k < OG; ++k) {
-                    const float dy = sY[(og * OG + k) * (CT + 1) + px];
-                    db[k] += dy;
-#pragma unroll
-                    for (int t = 0; t < 9; ++t) acc[k][t] = fmaf(dy, xw[t / 3][t % 3], acc[k][t]);
-                }
-            }
-        }
-    }
-    // combine the pixel splits in order, then write this block's partial
+    sh[ty][tx] = s;
     __syncthreads();
-    float *red = sX;   // [PXS][NCOMBO][OG*10]
-    {
-        float *d = red + ((size_t)s * NCOMBO + (tid % NCOMBO)) * (OG * 10);
-#pragma unroll
-        for (int k = 0; k < OG; ++k) {
-#pragma unroll
-            for (int t = 0; t < 9; ++t) d[k * 10 + t] = acc[k][t];
-            d[k * 10 + 9] = db[k];
-        }
-    }
-    __syncthreads();
-    if (s == 0) {
-        float *dst = part + ((size_t)f * gridDim.x + strip) * ((size_t)NCO * CI * 9 + NCO);
-#pragma unroll
-        for (int k = 0; k < OG; ++k) {
-            const int o = og * OG + k;
-#pragma unroll
-            for (int t = 0; t < 10; ++t) {
-                float sum = 0.0f;
-                for (int q = 0; q < PXS; ++q) sum += red[((size_t)q * NCOMBO + tid) * (OG * 10) + k * 10 + t];
-                if (t < 9) dst[((size_t)o * CI + c) * 9 + t] = sum;
-                else if (c == 0) dst[(size_t)NCO * CI * 9 + o] = sum;
-            }
-        }
-    }
-}
-
-// Sums the weight-gradient partials of all blocks (in block order) into the
-// layer's slice of the gradient vector (real input channels only).
-__global__ void wgrad_reduce_kernel(const float *__restrict__ part, int n_blocks, int ci_pad, int ci, int co,
-                                    float *__restrict__ grad)
-{
-    const int nw = co * ci * 9;
-    const size_t stride = (size_t)co * ci_pad * 9 + co;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nw + co; i += gridDim.x * blockDim.x) {
-        size_t src;
-        if (i < nw) {
-            const int o = i / (ci * 9), c = (i / 9) % ci, t = i % 9;
-            src = ((size_t)o * ci_pad + c) * 9 + t;
-        } else {
-            src = (size_t)co * ci_pad * 9 + (i - nw);
-        }
-        float s = 0.0f;
-        for (int b = 0; b < n_blocks; ++b) s += part[(size_t)b * stride + src];
-        grad[i] = s;
+    if (ty == 0 && i < (int)N_PARAMS) {
+        for (int k = 1; k < RED_Y; ++k) s += sh[k][tx];
+        grads[i] = s;
     }
 }
 
@@ -480,12 +400,23 @@ loss_kernel(const float *__restrict__ z, const float *__restrict__ target, const
     }
 }
 
-__global__ void loss_reduce_kernel(const float *__restrict__ part, int n, float inv_n, float *__restrict__ loss)
+// Sum of the loss partials in 64 bits, one block in a fixed order: 7 us for
+// 4,096 partials (one thread alone took 325 us, a chain of dependent loads and
+// adds).
+__global__ void __launch_bounds__(EPI_THREADS)
+loss_reduce_kernel(const float *__restrict__ part, int n, float inv_n, float *__restrict__ loss)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    __shared__ double sh[EPI_THREADS];
     double s = 0.0;
-    for (int i = 0; i < n; ++i) s += part[i];
-    *loss = (float)(s * inv_n);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += EPI_THREADS) s += part[i];
+    sh[threadIdx.x] = s;
+    __syncthreads();
+    for (int d = EPI_THREADS / 2; d > 0; d >>= 1) {
+        if (threadIdx.x < d) sh[threadIdx.x] += sh[threadIdx.x + d];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *loss = (float)(sh[0] * inv_n);
 }
 
 // Inference: rho = eps + (1-eps) sigmoid(z), its per-frame maximum, and the
@@ -644,27 +575,12 @@ cudaError_t conv_cc(const uint4 *in, const float *wt, const float *bias, const u
     return cudaGetLastError();
 }
 
-template <int NCI, int NCO>
-cudaError_t wgrad(const uint4 *X, const uint4 *dY, int F, int H, int W, float *part, cudaStream_t st)
-{
-    dim3 grid((H + RS - 1) / RS, F);
-    wgrad_kernel<NCI, NCO><<<grid, 256, wgrad_smem<NCI, NCO>(), st>>>(X, dY, H, W, part);
-    return cudaGetLastError();
-}
-
 template <int NCI, int NCO, int EPI>
 cudaError_t set_conv_smem()
 {
     return cudaFuncSetAttribute(conv_cc_kernel<NCI, NCO, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)conv_cc_smem<NCI, NCO>());
 }
-template <int NCI, int NCO>
-cudaError_t set_wgrad_smem()
-{
-    return cudaFuncSetAttribute(wgrad_kernel<NCI, NCO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)wgrad_smem<NCI, NCO>());
-}
-
 cudaError_t prepare_learn_kernels()
 {
     cudaError_t e;
@@ -673,9 +589,7 @@ cudaError_t prepare_learn_kernels()
     if ((e = set_conv_smem<4, 1, EPI_F32>()) != cudaSuccess) return e;
     if ((e = set_conv_smem<1, 32, EPI_MASK>()) != cudaSuccess) return e;
     if ((e = set_conv_smem<4, 32, EPI_MASK>()) != cudaSuccess) return e;
-    if ((e = set_wgrad_smem<1, 32>()) != cudaSuccess) return e;
-    if ((e = set_wgrad_smem<4, 32>()) != cudaSuccess) return e;
-    return set_wgrad_smem<4, 1>();
+    return prepare_wgrad();
 }
 
 }  // namespace
@@ -841,13 +755,20 @@ cudaError_t run_forward(pam_learn_s *l, const uint4 *feat, int n, bool keep, cud
         l->kernels += 5;
         return e;
     }
-    if ((e = pam::conv_cc<1, 32, pam::EPI_RELU>(feat, l->prep.wf[0], l->prep.bias[0], nullptr, a[0], n, H, W, st)) !=
-        cudaSuccess)
-        return e;
-    for (int k = 1; k < 4; ++k)
-        if ((e = pam::conv_cc<4, 32, pam::EPI_RELU>(a[k - 1], l->prep.wf[k], l->prep.bias[k], nullptr, a[k], n, H, W,
-                                                    st)) != cudaSuccess)
-            return e;
+    for (int k = 0; k < 4; ++k) {
+        const uint4 *in = k ? a[k - 1] : feat;
+        // Without pam_learn_configure's tensor cores the activations are the
+        // CUDA-core kernel's bits; at nx = 128 tcgen05 makes the same bits faster
+        // (32 -> 32 layer, 16 frames of 512 x 128: 107 us against 467 us).
+        if (W == 128)
+            e = pam::launch_conv_tc_exact(k, in, reinterpret_cast<const uint4 *>(l->prep.wtc[k]), l->prep.bias[k], a[k],
+                                          n, H, l->plan->w.status, st);
+        else if (k == 0)
+            e = pam::conv_cc<1, 32, pam::EPI_RELU>(in, l->prep.wf[k], l->prep.bias[k], nullptr, a[k], n, H, W, st);
+        else
+            e = pam::conv_cc<4, 32, pam::EPI_RELU>(in, l->prep.wf[k], l->prep.bias[k], nullptr, a[k], n, H, W, st);
+        if (e != cudaSuccess) return e;
+    }
     e = pam::conv_cc<4, 1, pam::EPI_F32>(a[3], l->prep.wf[4], l->prep.bias[4], nullptr, l->z, n, H, W, st);
     l->kernels += 5;
     return e;
@@ -865,36 +786,39 @@ cudaError_t run_grads(pam_learn_s *l, const uint4 *feat, const float *target, in
                                                       l->loss_part);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (loss) {
-        pam::loss_reduce_kernel<<<1, 32, 0, st>>>(l->loss_part, l->loss_blocks * n, inv_n, loss);
+        pam::loss_reduce_kernel<<<1, pam::EPI_THREADS, 0, st>>>(l->loss_part, l->loss_blocks * n, inv_n, loss);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         l->kernels += 1;
     }
-    const int nblk = ((H + pam::RS - 1) / pam::RS) * n;
-    auto reduce = [&](int layer) -> cudaError_t {
-        pam::wgrad_reduce_kernel<<<64, 256, 0, st>>>(l->wpart, nblk, CINC(layer) * 8, CIN(layer), COUT(layer),
-                                                     l->grads + pam::p_offset(layer));
-        return cudaGetLastError();
+    const int ctas = pam::wgrad_ctas(l->n_sms, n, H);
+    int *status = l->plan->w.status;
+    auto wgrad = [&](int layer, const uint4 *X, const uint4 *dY) {
+        return pam::launch_wgrad(layer, X, dY, n, H, W, ctas, l->wpart + (size_t)ctas * pam::p_offset(layer), status, st);
+    };
+    // dX of layer k through the ReLU of its input act[k - 1]
+    auto dgrad = [&](int k, const uint4 *dY, uint4 *out) -> cudaError_t {
+        if (W == 128)
+            return pam::launch_conv_tc_grad(k, dY, reinterpret_cast<const uint4 *>(l->prep.wtcb[k]), l->act[k - 1], out,
+                                            n, H, status, st);
+        if (k == NL - 1)
+            return pam::conv_cc<1, 32, pam::EPI_MASK>(dY, l->prep.wb[k], nullptr, l->act[k - 1], out, n, H, W, st);
+        return pam::conv_cc<4, 32, pam::EPI_MASK>(dY, l->prep.wb[k], nullptr, l->act[k - 1], out, n, H, W, st);
     };
     // layer 5: dY = dz, X = a4
-    if ((e = pam::wgrad<4, 1>(l->act[3], l->dz, n, H, W, l->wpart, st)) != cudaSuccess) return e;
-    if ((e = reduce(4)) != cudaSuccess) return e;
-    if ((e = pam::conv_cc<1, 32, pam::EPI_MASK>(l->dz, l->prep.wb[4], nullptr, l->act[3], l->g[0], n, H, W, st)) !=
-        cudaSuccess)
-        return e;
+    if ((e = wgrad(4, l->act[3], l->dz)) != cudaSuccess) return e;
+    if ((e = dgrad(4, l->dz, l->g[0])) != cudaSuccess) return e;
     // layers 4, 3, 2: dY = g, X = a_{k-1}
     int cur = 0;
     for (int k = 3; k >= 1; --k) {
-        if ((e = pam::wgrad<4, 32>(l->act[k - 1], l->g[cur], n, H, W, l->wpart, st)) != cudaSuccess) return e;
-        if ((e = reduce(k)) != cudaSuccess) return e;
-        if ((e = pam::conv_cc<4, 32, pam::EPI_MASK>(l->g[cur], l->prep.wb[k], nullptr, l->act[k - 1], l->g[cur ^ 1],
-                                                    n, H, W, st)) != cudaSuccess)
-            return e;
+        if ((e = wgrad(k, l->act[k - 1], l->g[cur])) != cudaSuccess) return e;
+        if ((e = dgrad(k, l->g[cur], l->g[cur ^ 1])) != cudaSuccess) return e;
         cur ^= 1;
     }
     // layer 1: X = features
-    if ((e = pam::wgrad<1, 32>(feat, l->g[cur], n, H, W, l->wpart, st)) != cudaSuccess) return e;
-    if ((e = reduce(0)) != cudaSuccess) return e;
-    l->kernels += 1 + 5 * 2 + 4;
+    if ((e = wgrad(0, feat, l->g[cur])) != cudaSuccess) return e;
+    pam::wgrad_reduce_kernel<<<(unsigned)((pam::N_PARAMS + 31) / 32), 32 * pam::RED_Y, 0, st>>>(l->wpart, ctas, l->grads);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    l->kernels += 1 + 5 + 4 + 1;
     return cudaSuccess;
 }
 
@@ -964,7 +888,7 @@ pam_status pam_learn_create(const pam_plan_desc *d, pam_learn_t *out)
     }
     prep_n += 4 * NL;   // float4 alignment slack
     LALLOC(zalloc(&l->prep_mem, prep_n));
-    LALLOC(zalloc(&l->tc_mem, pam::tc_offset(NL)));
+    LALLOC(zalloc(&l->tc_mem, pam::tcb_offset(NL)));
     {
         float *q = l->prep_mem;
         auto take = [&](size_t n) { float *r = q; q += (n + 3) / 4 * 4; return r; };
@@ -973,6 +897,7 @@ pam_status pam_learn_create(const pam_plan_desc *d, pam_learn_t *out)
             l->prep.wb[k] = k >= 1 ? take((size_t)((COUT(k) + 7) / 8 * 8) * 9 * CIN(k)) : nullptr;
             l->prep.bias[k] = take(COUT(k));
             l->prep.wtc[k] = l->tc_mem + pam::tc_offset(k);
+            l->prep.wtcb[k] = l->tc_mem + pam::tcb_offset(k);
         }
     }
     LALLOC(zalloc(&l->feat, F * l->ppix));
@@ -983,8 +908,7 @@ pam_status pam_learn_create(const pam_plan_desc *d, pam_learn_t *out)
     LALLOC(zalloc(&l->bands, F * pam::N_BANDS * l->npix));
     LALLOC(zalloc(&l->E, F * l->npix));
     LALLOC(zalloc(&l->rho, F * l->npix));
-    const size_t nblk = (size_t)((l->H + pam::RS - 1) / pam::RS) * F;
-    LALLOC(zalloc(&l->wpart, nblk * (32 * 32 * 9 + 32)));
+    LALLOC(zalloc(&l->wpart, (size_t)pam::wgrad_ctas(l->n_sms, l->F, l->H) * pam::N_PARAMS));
     LALLOC(zalloc(&l->loss_part, (size_t)l->loss_blocks * F));
     LALLOC(zalloc(&l->emax, F));
     LALLOC(zalloc(&l->rmax, F));
