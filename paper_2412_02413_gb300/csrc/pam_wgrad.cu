@@ -1,32 +1,39 @@
 // pam_wgrad.cu -- weight gradients of the 3x3 convolutions of the learned
-// NCC-weight network on the tensor cores (mma.sync, BF16 operands, FP32 sums).
+// NCC-weight network on the tensor cores (tcgen05, BF16 operands, FP32 sums).
 //
 // dW[o][c][u][v] = sum_{f,i,j} dY[f][o][i][j] X[f][c][i+u-1][j+v-1], db[o] = sum dY
-// is, per output row, a GEMM whose K runs over the row's pixels: M = (tap,
-// input channel), N = output channel. Activations and gradients are stored
-// chunked and padded, BF16 [C/8][H+2][W+2][8], so the 8 channels of one chunk
-// at 8 consecutive pixels are an 8 x 8 matrix of 16-byte rows that
-// ldmatrix.trans reads as (channel, pixel) fragments; a tap's column shift
-// only moves the row addresses by 16 bytes per pixel and its row shift picks
-// another staged row, so nothing is rearranged in memory.
-//
-// Why mma.sync and not tcgen05: N is 32 (8 for the last layer), and a tcgen05
-// MMA of M = 128, N = 32 reads its 4 KB A tile from shared memory in 32 clocks
-// for 16 clocks of tensor work, so both reach about the same rate here, near
-// the time the two tensors take from HBM, and this form serves every width.
+// is, per output row i and column shift v, a GEMM whose K runs over the row's
+// pixels: M = (row shift u, input channel c), N = output channel o. Activations
+// and gradients are stored chunked and padded, BF16 [C/8][H+2][W+2][8], so a row
+// of one chunk copied as it is into shared memory is a column of 8 x 8 core
+// matrices of the MN-major layout without swizzle: 8 channels in 16 contiguous
+// bytes, 16 bytes per pixel along K (LBO: the next 8 pixels, 128 bytes). The
+// next 8 channels are the next chunk and, past a row's last chunk, the next
+// staged row, at one stride (SBO): staged rows i, i+1, i+2 are the operand of the
+// three row shifts at once, and a column shift moves the start address by 16
+// bytes. Nothing is rearranged in memory.
 //
 // Work: one CTA per SM takes an equal contiguous share of the batch's rows
-// (frame after frame); thread 0 stages each input row (three output rows use
-// it) and each dY row once through two rings of bulk copies, so that 12 warps
-// keep up to 168 registers each (a 13th, a producer of its own, would leave
-// 128 and spill). The warps are GROUPS x SPLITS: a group owns a part of the (tap, chunk) tiles, a
-// split every SPLITS-th group of 16 pixels of the row. At the end the splits
-// are added in order and the CTA writes one partial; wgrad_reduce_kernel adds the
-// CTAs' partials in order, so results do not depend on timing.
+// (frame after frame). Warp 0 stages each input row (three output rows use it)
+// and each dY row once, by bulk copies into two rings; warps 1-3 issue one column
+// shift's W / 16 MMAs (M = 128, N = 32 or 16, K = 16) per output row each; warps 4-7
+// add up db from the staged dY rows and, every FLUSH rows, add the accumulators of
+// the three column shifts to FP32 sums in registers, while the MMAs go on into a
+// second set of accumulators (a chain of FLUSH W / 16 tensor-core steps keeps the
+// rounding of the accumulators, which the hardware truncates, below that of the
+// FP32 sums). The CTA writes one partial; wgrad_reduce_kernel adds the CTAs'
+// partials in order, so results do not depend on timing.
 //
-// Measured (GB300, 16 frames of 512 x 128): 97 us for 32 -> 32 channels, 56
-// and 55 us for the first and last layers, against 689, 197 and 86 us on the
-// CUDA cores; bound by the mma.sync rate.
+// A window of 16 groups of 8 channels is more than the three rows: the groups
+// past them read whatever the following slots hold, which only reaches
+// accumulator rows (or, with one dY chunk, columns) that nobody reads.
+//
+// Measured (GB300, 16 frames of 512 x 128): 47 us for 32 -> 32 channels, 42 us for
+// the first and last layers, where one issuing warp took 61 us, mma.sync 97 us (its
+// rate) and the CUDA cores 689 us. Bound by the hand-offs of a row (0.8 us):
+// halving the MMAs, dropping the db sums or deepening the rings changes it by less
+// than 5%, and DRAM runs at 3.1 TB/s. One MMA of N = 96 per 16 pixels, with dY
+// staged once per column shift, took 61 us (three times the copies).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -38,271 +45,264 @@ namespace {
 
 using namespace ptx;
 
-constexpr int NSX = 8, NSY = 6;   // ring slots of input rows and dY rows (NSY >= NSX - 2)
+constexpr int NSX = 8, NSY = 6;    // ring slots of input rows and dY rows (NSY >= NSX - 2)
+constexpr int FLUSH = 4;           // output rows per accumulator set
+constexpr int THREADS = 256;
+constexpr int GROUPS = 16;         // 8-channel groups of M = 128
 
-// NCI input chunks, NCY dY chunks (of 8 channels). TILES m16 tiles of two
-// (tap, chunk) blocks each.
+// NCI input chunks, NCY dY chunks (of 8 channels).
 template <int NCI, int NCY>
 struct WG {
-    static constexpr int BLOCKS = 9 * NCI;
-    static constexpr int TILES = (BLOCKS + 1) / 2;
-    static constexpr int GROUPS = TILES * NCY > 40 ? 3 : 1;   // accumulators per thread: 4 TILES NCY / GROUPS
-    static constexpr int SPLITS = GROUPS == 3 ? 4 : 8;
-    static constexpr int TPG = TILES / GROUPS;
-    static_assert(TPG * GROUPS == TILES, "tiles divide among the groups");
-    static constexpr int WARPS = GROUPS * SPLITS;
-    static constexpr int THREADS = 32 * WARPS;
-    static constexpr int NR = (TPG + 1) * NCY * 4;     // floats per thread of the split reduction (tiles, db)
-    static constexpr size_t ring(int W) { return (size_t)(NSX * NCI + NSY * NCY) * (W + 2) * 16; }
-    static constexpr size_t red() { return (size_t)GROUPS * NR * 32 * 4; }
-    static constexpr size_t smem(int W) { return 256 + (ring(W) > red() ? ring(W) : red()); }
+    static constexpr int NB = NCY == 1 ? 16 : 8 * NCY;     // GEMM columns (at least 16 for M = 128)
+    static constexpr int VROWS = 3 * NCI * 8;              // accumulator rows in use
+    // input ring: NSX slots, the first two again behind the last (a window of
+    // three rows is contiguous from any slot), and room for the rest of the window
+    static constexpr int XSLOTS = NSX + 2;
+    static constexpr int XCHUNKS = (NSX - 1) * NCI + GROUPS > XSLOTS * NCI ? (NSX - 1) * NCI + GROUPS : XSLOTS * NCI;
+    static constexpr int YCHUNKS = NSY * NCY + 1;          // the second column group of NCY = 1 reads one further
+    static constexpr size_t smem(int W) { return 1024 + (size_t)(XCHUNKS + YCHUNKS) * (W + 2) * 16; }
 };
 
-__device__ __forceinline__ void ldsm4t(unsigned (&r)[4], unsigned addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(addr)
-                 : "memory");
-}
-__device__ __forceinline__ void ldsm2t(unsigned (&r)[2], unsigned addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n"
-                 : "=r"(r[0]), "=r"(r[1])
-                 : "r"(addr)
-                 : "memory");
-}
-__device__ __forceinline__ void mma16816(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1)
-{
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-                 "{%0,%1,%2,%3};\n"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
+// kind::f16, FP32 accumulators, BF16 operands, both MN-major
+constexpr unsigned idesc_mn(int n) { return umma_idesc(false, 128, n) | (1u << 15) | (1u << 16); }
 
 // part: [gridDim.x][CO * CI * 9 + CO] partial sums in the parameter layout of
 // the layer (w[o][c][3][3], then b[o]; CI, CO real channels).
 template <int NCI, int NCY>
-__global__ void __launch_bounds__(WG<NCI, NCY>::THREADS, 1)
+__global__ void __launch_bounds__(THREADS, 1)
 wgrad_tc_kernel(const uint4 *__restrict__ X, const uint4 *__restrict__ dY, int F, int H, int W, int CI, int CO,
                 float *__restrict__ part, int *__restrict__ status)
 {
     using G = WG<NCI, NCY>;
-    constexpr int TPG = G::TPG;
-    extern __shared__ __align__(128) uint8_t sm[];
+    constexpr int NB = G::NB;
+    extern __shared__ __align__(1024) uint8_t sm[];
     uint64_t *xfull = reinterpret_cast<uint64_t *>(sm);   // [NSX] input row has landed
-    uint64_t *xfree = xfull + NSX;                        // [NSX] every warp is done with it
-    uint64_t *yfull = xfree + NSX, *yfree = yfull + NSY;  // [NSY] the same for dY rows
+    uint64_t *xfree = xfull + NSX;                        // [NSX] the MMAs (3 commits) that read it are done
+    uint64_t *yfull = xfree + NSX, *yfree = yfull + NSY;  // [NSY] dY rows: 3 MMA warps and the 4 db warps
+    uint64_t *afull = yfree + NSY, *aempty = afull + 2;   // [2] accumulator sets
+    uint64_t *dbar = aempty + 2;                          // [3] drain
+    unsigned *tslot = reinterpret_cast<unsigned *>(dbar + 3);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(tslot + 1);
+    float *sdb = reinterpret_cast<float *>(sm + 512);     // [4 warps][32] db of each warp's pixels
     const unsigned CHB = (unsigned)(W + 2) * 16u;         // one row of one chunk
-    uint8_t *sX = sm + 256, *sY = sX + (size_t)NSX * NCI * CHB;
+    uint8_t *sX = sm + 1024, *sY = sX + (size_t)G::XCHUNKS * CHB;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (tid == 0) {
+    if (warp == 0) tmem_alloc(tslot, 256u);
+    if (tid == 32) {
         for (int s = 0; s < NSX; ++s) {
             mbar_init(&xfull[s], 1);
-            mbar_init(&xfree[s], G::WARPS);
+            mbar_init(&xfree[s], 3);
         }
         for (int s = 0; s < NSY; ++s) {
             mbar_init(&yfull[s], 1);
-            mbar_init(&yfree[s], G::WARPS);
+            mbar_init(&yfree[s], 7);
         }
+        for (int t = 0; t < 2; ++t) {
+            mbar_init(&afull[t], 3);
+            mbar_init(&aempty[t], 4);
+        }
+        for (int v = 0; v < 3; ++v) mbar_init(&dbar[v], 1);
+        *abort_flag = 0;
         mbar_fence_init();
     }
+    tc_fence_before();
     __syncthreads();
+    tc_fence_after();
+    const unsigned tmem = *tslot;
 
+    // Bounded wait that also gives up when another warp has.
+    auto wait = [&](uint64_t *b, unsigned parity) -> bool {
+        if (mbar_try_wait_sleep(b, parity)) return true;
+        const long long t0 = clock64();
+        while (!mbar_try_wait_sleep(b, parity)) {
+            if (*abort_flag) return false;
+            if (clock64() - t0 > (1ll << 31)) {
+                *abort_flag = 1;
+                atomicOr(status, 1);
+                return false;
+            }
+        }
+        return true;
+    };
+
+    // The share's rows, in segments of one frame: n output rows from row a of
+    // frame f use n + 2 staged input rows (counted by nx) and n dY rows (ny).
     const long long T = (long long)F * H;
     const long long r0 = T * blockIdx.x / gridDim.x, r1 = T * (blockIdx.x + 1) / gridDim.x;
     const int HP = H + 2, WP = W + 2;
+    unsigned nx = 0, ny = 0;
     bool ok = true;
 
-    // Producer (thread 0): the rows of each segment (one frame's part of the
-    // share) in order; input row k of a segment comes with the dY row of output
-    // row k - 2. `seen` is the first input row that the thread's own warp still
-    // needs: at most NSX - 1 rows from there are staged, so the slot to fill held
-    // a row that the other warps finished two of their rows ago.
-    unsigned px = 0, py = 0;      // rows issued
-    long long pr = r0;            // next segment's first row
-    int pf = 0, pa = 0, pn = 0, pk = 0;
-    auto issue = [&](unsigned seen) {
-        while (ok && px < seen + NSX - 1) {
-            if (pk == (pn ? pn + 2 : 0)) {   // next segment
-                if (pr >= r1) return;
-                pf = (int)(pr / H);
-                pa = (int)(pr - (long long)pf * H);
-                pn = (int)min((long long)(H - pa), r1 - pr);
-                pr += pn;
-                pk = 0;
+    if (warp == 0) {
+        // ---------------- producer: lane c copies chunk c ----------------
+        for (long long r = r0; r < r1 && ok;) {
+            const int f = (int)(r / H), a = (int)(r - (long long)f * H);
+            const int n = (int)min((long long)(H - a), r1 - r);
+            for (int k = 0; k < n + 2; ++k) {
+                const unsigned s = nx % NSX;
+                const bool twice = s < 2;   // again behind the last slot
+                if (nx >= NSX) ok = __all_sync(0xffffffffu, wait(&xfree[s], (nx / NSX - 1) & 1u));
+                if (!ok) break;
+                if (lane == 0) mbar_expect_tx(&xfull[s], (twice ? 2u : 1u) * NCI * CHB);
+                __syncwarp();
+                if (lane < (twice ? 2 : 1) * NCI) {
+                    const int c = lane % NCI;
+                    bulk_g2s(sX + (size_t)((s + (lane >= NCI ? NSX : 0)) * NCI + c) * CHB,
+                             X + (((size_t)f * NCI + c) * HP + a + k) * WP, CHB, &xfull[s]);
+                }
+                ++nx;
+                if (k < 2) continue;
+                const unsigned t = ny % NSY;   // dY row a + k - 2, padded row + 1
+                if (ny >= NSY) ok = __all_sync(0xffffffffu, wait(&yfree[t], (ny / NSY - 1) & 1u));
+                if (!ok) break;
+                if (lane == 0) mbar_expect_tx(&yfull[t], NCY * CHB);
+                __syncwarp();
+                if (lane < NCY)
+                    bulk_g2s(sY + (size_t)(t * NCY + lane) * CHB, dY + (((size_t)f * NCY + lane) * HP + a + k - 1) * WP,
+                             CHB, &yfull[t]);
+                ++ny;
             }
-            const unsigned s = px % NSX;
-            if (px >= NSX) ok = mbar_wait(&xfree[s], (px / NSX - 1) & 1u);
-            if (!ok) return;
-            mbar_expect_tx(&xfull[s], NCI * CHB);
-            for (int c = 0; c < NCI; ++c)
-                bulk_g2s(sX + (size_t)(s * NCI + c) * CHB, X + (((size_t)pf * NCI + c) * HP + pa + pk) * WP, CHB,
-                         &xfull[s]);
-            ++px;
-            if (++pk < 3) continue;
-            const unsigned t = py % NSY;         // dY row pa + pk - 3, padded row + 1
-            if (py >= NSY) ok = mbar_wait(&yfree[t], (py / NSY - 1) & 1u);
-            if (!ok) return;
-            mbar_expect_tx(&yfull[t], NCY * CHB);
-            for (int c = 0; c < NCY; ++c)
-                bulk_g2s(sY + (size_t)(t * NCY + c) * CHB, dY + (((size_t)pf * NCY + c) * HP + pa + pk - 2) * WP, CHB,
-                         &yfull[t]);
-            ++py;
+            r += n;
         }
-    };
-
-    const int grp = warp / G::SPLITS, split = warp % G::SPLITS;
-    const bool with_db = grp == 0;
-    float acc[TPG + 1][NCY][4];   // the last tile's rows are all sum_k dY (a tile of ones), for db
-#pragma unroll
-    for (int t = 0; t <= TPG; ++t)
-#pragma unroll
-        for (int n = 0; n < NCY; ++n)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) acc[t][n][k] = 0.0f;
-
-    {
-        // Row of the lane's 8 x 8 matrix in an ldmatrix.x4: matrices are (block 0,
-        // pixels 0-7), (block 1, 0-7), (block 0, 8-15), (block 1, 8-15) for A and
-        // (chunk n, 0-7), (n, 8-15), (n + 1, 0-7), (n + 1, 8-15) for B.
-        const int mi = lane >> 3;
-        const unsigned a_px = (unsigned)((lane & 7) + 8 * (mi >> 1)), b_px = (unsigned)((lane & 7) + 8 * (mi & 1));
-        // byte offset of the lane's block inside the three staged rows: row shift u
-        // (a slot index, resolved per row), and chunk and column shift
-        int a_u[TPG];
-        unsigned a_off[TPG];
-#pragma unroll
-        for (int t = 0; t < TPG; ++t) {
-            int blk = 2 * (grp * TPG + t) + (mi & 1);
-            if (blk >= G::BLOCKS) blk = G::BLOCKS - 1;   // odd count: the spare rows are dropped at the end
-            const int tap = blk / NCI, c = blk % NCI;
-            a_u[t] = tap / 3;
-            a_off[t] = (unsigned)c * CHB + ((unsigned)(tap % 3) + a_px) * 16u;
+        if (lane == 0) {
+            if (*abort_flag) {   // the copies in flight land before the CTA exits
+                for (unsigned k = nx < NSX ? 0 : nx - NSX; k < nx; ++k) mbar_wait(&xfull[k % NSX], (k / NSX) & 1u);
+                for (unsigned k = ny < NSY ? 0 : ny - NSY; k < ny; ++k) mbar_wait(&yfull[k % NSY], (k / NSY) & 1u);
+            }
         }
-        const unsigned b_off = (NCY > 1 ? (unsigned)(mi >> 1) * CHB : 0u) + (1u + b_px) * 16u;   // dY has the border too
-        const unsigned ones[4] = {0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u};
+        __syncwarp();
+    } else if (warp < 4) {
+        // ---------------- MMA issue, column shift v ----------------
+        const int v = warp - 1;
         const unsigned xb = smem_u32(sX), yb = smem_u32(sY);
-        unsigned nx = 0, ny = 0;   // rows of earlier segments
+        const int rows = (int)(r1 - r0);
+        int done = 0;
+        bool any = false;
         for (long long r = r0; r < r1 && ok;) {
             const int a = (int)(r % H);
             const int n = (int)min((long long)(H - a), r1 - r);
-            for (int i = 0; i < n && ok; ++i) {
-                if (tid == 0) issue(nx + (unsigned)i);
+            for (int i = 0; i < n; ++i) {
                 // input rows nx + i .. nx + i + 2 (the first two were waited for by earlier rows)
-                for (int k = i == 0 ? 0 : 2; k < 3 && ok; ++k)
-                    ok = mbar_wait(&xfull[(nx + i + k) % NSX], ((nx + i + k) / NSX) & 1u);
+                for (unsigned k = i == 0 ? 0u : 2u; k < 3u && ok; ++k)
+                    ok = wait(&xfull[(nx + i + k) % NSX], ((nx + i + k) / NSX) & 1u);
                 const unsigned y = ny + (unsigned)i;
-                if (ok) ok = mbar_wait(&yfull[y % NSY], (y / NSY) & 1u);
+                if (ok) ok = wait(&yfull[y % NSY], (y / NSY) & 1u);
+                const int set = done / FLUSH, t = set & 1;
+                if (ok && done % FLUSH == 0 && set >= 2) ok = wait(&aempty[t], (unsigned)((set >> 1) - 1) & 1u);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
-                unsigned xrow[3];
-#pragma unroll
-                for (int u = 0; u < 3; ++u) xrow[u] = xb + ((nx + (unsigned)(i + u)) % NSX) * (NCI * CHB);
-                const unsigned yrow = yb + (y % NSY) * (NCY * CHB) + b_off;
-                for (int ks = split; ks < W / 16; ks += G::SPLITS) {
-                    unsigned b[NCY][2];
-                    if constexpr (NCY > 1) {
-#pragma unroll
-                        for (int q = 0; q < NCY; q += 2) {
-                            unsigned v[4];
-                            ldsm4t(v, yrow + (unsigned)q * CHB + (unsigned)ks * 256u);
-                            b[q][0] = v[0]; b[q][1] = v[1]; b[q + 1][0] = v[2]; b[q + 1][1] = v[3];
-                        }
-                    } else {
-                        ldsm2t(b[0], yrow + (unsigned)ks * 256u);
-                    }
-#pragma unroll
-                    for (int t = 0; t < TPG; ++t) {
-                        unsigned av[4];
-                        const unsigned row = a_u[t] == 0 ? xrow[0] : a_u[t] == 1 ? xrow[1] : xrow[2];
-                        ldsm4t(av, row + a_off[t] + (unsigned)ks * 256u);
-#pragma unroll
-                        for (int q = 0; q < NCY; ++q) mma16816(acc[t][q], av, b[q][0], b[q][1]);
-                    }
-                    if (with_db) {
-#pragma unroll
-                        for (int q = 0; q < NCY; ++q) mma16816(acc[TPG][q], ones, b[q][0], b[q][1]);
-                    }
+                tc_fence_after();
+                const unsigned arow = xb + ((nx + (unsigned)i) % NSX) * (NCI * CHB) + (unsigned)v * 16u;
+                const unsigned brow = yb + (y % NSY) * (NCY * CHB) + 16u;   // dY has the border too
+                const uint64_t da0 = umma_desc(arow, 128, CHB), db0 = umma_desc(brow, 128, CHB);
+#pragma unroll 8
+                for (int ks = 0; ks < W / 16; ++ks)
+                    umma_elect(tmem + (unsigned)((t * 3 + v) * NB), da0 + (uint64_t)(ks * 16), db0 + (uint64_t)(ks * 16),
+                               idesc_mn(NB), (done % FLUSH || ks) ? 1u : 0u);
+                any = true;
+                umma_commit_elect(&xfree[(nx + i) % NSX]);
+                if (i == n - 1) {   // the segment's last two rows are not used again
+                    umma_commit_elect(&xfree[(nx + i + 1) % NSX]);
+                    umma_commit_elect(&xfree[(nx + i + 2) % NSX]);
                 }
-                __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(&xfree[(nx + i) % NSX]);
-                    if (i == n - 1) {   // the segment's last two rows are not used again
-                        mbar_arrive(&xfree[(nx + i + 1) % NSX]);
-                        mbar_arrive(&xfree[(nx + i + 2) % NSX]);
-                    }
-                    mbar_arrive(&yfree[y % NSY]);
-                }
+                umma_commit_elect(&yfree[y % NSY]);
+                ++done;
+                if (done % FLUSH == 0 || done == rows) umma_commit_elect(&afull[t]);
             }
             nx += (unsigned)n + 2u;
             ny += (unsigned)n;
             r += n;
         }
-        if (!ok && lane == 0) atomicOr(status, 1);
-    }
-    if (__syncthreads_or(!ok)) {
-        if (tid == 0) {   // the copies in flight land before the CTA exits
-            for (unsigned k = px < NSX ? 0 : px - NSX; k < px; ++k) mbar_wait(&xfull[k % NSX], (k / NSX) & 1u);
-            for (unsigned k = py < NSY ? 0 : py - NSY; k < py; ++k) mbar_wait(&yfull[k % NSY], (k / NSY) & 1u);
+        if (!ok && any && lane == 0) {
+            umma_commit(&dbar[v]);
+            mbar_wait(&dbar[v], 0);
         }
-        return;
-    }
-    // every row has been read: the rings' memory is free
-
-    // the splits' sums added to split 0's, in order
-    float *red = reinterpret_cast<float *>(sX) + (size_t)grp * (G::NR * 32);
-    for (int s = 1; s < G::SPLITS; ++s) {
-        if (split == s) {
+        __syncwarp();
+    } else {
+        // ---------------- sums ----------------
+        const int quarter = warp & 3, ctid = tid - 128;
+        float sum[3][NB == 16 ? 1 : NB];   // NCY = 1 has one real output channel
+        constexpr int NO = NB == 16 ? 1 : NB;
 #pragma unroll
-            for (int t = 0; t <= TPG; ++t)
+        for (int v = 0; v < 3; ++v)
 #pragma unroll
-                for (int q = 0; q < NCY; ++q)
+            for (int o = 0; o < NO; ++o) sum[v][o] = 0.0f;
+        float db[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        // db: this thread's chunk and pixels (128 / NCY threads per chunk)
+        const int ch = NCY == 1 ? 0 : ctid & (NCY - 1), p0 = ctid / NCY;
+        const int rows = (int)(r1 - r0);
+        for (int y = 0; y < rows; ++y) {
+            if (!__all_sync(0xffffffffu, wait(&yfull[y % NSY], (unsigned)(y / NSY) & 1u))) break;
+            const uint4 *row = reinterpret_cast<const uint4 *>(sY + (size_t)((y % NSY) * NCY + ch) * CHB) + 1;
+            for (int p = p0; p < W; p += 128 / NCY) {
+                const uint4 q = row[p];
+                const unsigned w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) red[((t * NCY + q) * 4 + k) * 32 + lane] = acc[t][q][k];
-        }
-        __syncthreads();
-        if (split == 0) {
-#pragma unroll
-            for (int t = 0; t <= TPG; ++t)
-#pragma unroll
-                for (int q = 0; q < NCY; ++q)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) acc[t][q][k] += red[((t * NCY + q) * 4 + k) * 32 + lane];
-        }
-        __syncthreads();
-    }
-    if (split != 0) return;
-    // fragment (k): block row lane / 4 (+ 8 for k >= 2: the tile's second block), column 2 (lane % 4) + (k & 1)
-    float *dst = part + (size_t)blockIdx.x * ((size_t)CO * CI * 9 + CO);
-    const int row = lane >> 2, col = 2 * (lane & 3);
-#pragma unroll
-    for (int t = 0; t < TPG; ++t)
-#pragma unroll
-        for (int q = 0; q < NCY; ++q)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int blk = 2 * (grp * TPG + t) + (k >> 1);
-                const int tap = blk / NCI, c = (blk % NCI) * 8 + row, o = q * 8 + col + (k & 1);
-                if (blk < G::BLOCKS && c < CI && o < CO) dst[((size_t)o * CI + c) * 9 + tap] = acc[t][q][k];
+                for (int k = 0; k < 4; ++k) {
+                    db[2 * k] += __uint_as_float(w[k] << 16);
+                    db[2 * k + 1] += __uint_as_float(w[k] & 0xFFFF0000u);
+                }
             }
-    if (with_db && row == 0) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&yfree[y % NSY]);
+            if ((y + 1) % FLUSH != 0 && y + 1 != rows) continue;
+            const int set = y / FLUSH, t = set & 1;
+            if (!__all_sync(0xffffffffu, wait(&afull[t], (unsigned)(set >> 1) & 1u))) break;
+            tc_fence_after();
+            const unsigned ta = tmem + (unsigned)(t * 3 * NB) + ((unsigned)(32 * quarter) << 16);
 #pragma unroll
-        for (int q = 0; q < NCY; ++q)
+            for (int v = 0; v < 3; ++v) {
+                if constexpr (NB == 32) {
+                    unsigned q[32];
+                    tmem_ld32(ta + (unsigned)(v * NB), q);
+                    tmem_wait_ld();
 #pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const int o = q * 8 + col + k;
-                if (o < CO) dst[(size_t)CO * CI * 9 + o] = acc[TPG][q][k];
+                    for (int o = 0; o < 32; ++o) sum[v][o] += __uint_as_float(q[o]);
+                } else {
+                    float q[4];
+                    tmem_ld4(ta + (unsigned)(v * NB), q);
+                    tmem_wait_ld();
+                    sum[v][0] += q[0];
+                }
             }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&aempty[t]);
+        }
+        // accumulator row 8 NCI u + c: this thread's (u, c)
+        float *dst = part + (size_t)blockIdx.x * ((size_t)CO * CI * 9 + CO);
+        const int m = 32 * quarter + lane, u = m / (8 * NCI), c = m % (8 * NCI);
+        if (!*abort_flag && m < G::VROWS && c < CI) {
+#pragma unroll
+            for (int v = 0; v < 3; ++v)
+#pragma unroll
+                for (int o = 0; o < NO; ++o)
+                    if (o < CO) dst[((size_t)o * CI + c) * 9 + 3 * u + v] = sum[v][o];
+        }
+        // db: lanes of one chunk, then the four warps in order
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+#pragma unroll
+            for (int d = 16; d >= NCY; d >>= 1) db[k] += __shfl_xor_sync(0xffffffffu, db[k], d);
+        if (lane < NCY)
+#pragma unroll
+            for (int k = 0; k < 8; ++k) sdb[(warp - 4) * 32 + lane * 8 + k] = db[k];
     }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 0) tmem_dealloc(tmem, 256u);
+    if (!*abort_flag && tid < CO && tid < 32)
+        part[(size_t)blockIdx.x * ((size_t)CO * CI * 9 + CO) + (size_t)CO * CI * 9 + tid] =
+            ((sdb[tid] + sdb[32 + tid]) + sdb[64 + tid]) + sdb[96 + tid];
 }
 
 template <int NCI, int NCY>
 cudaError_t launch_t(const uint4 *X, const uint4 *dY, int F, int H, int W, int CI, int CO, int ctas, float *part,
                      int *status, cudaStream_t st)
 {
-    using G = WG<NCI, NCY>;
-    wgrad_tc_kernel<NCI, NCY><<<ctas, G::THREADS, G::smem(W), st>>>(X, dY, F, H, W, CI, CO, part, status);
+    static_assert(WG<NCI, NCY>::smem(128) <= 232448, "shared memory of the weight gradient");
+    wgrad_tc_kernel<NCI, NCY><<<ctas, THREADS, WG<NCI, NCY>::smem(W), st>>>(X, dY, F, H, W, CI, CO, part, status);
     return cudaGetLastError();
 }
 
