@@ -25,7 +25,7 @@
 // One CTA per (16-row strip, frame), 6 warps:
 //   warp 0: bulk copies of the strip's 18 input rows through a ring of 6 slots;
 //   warp 1: the MMA chain of each output row (one elected lane issues);
-//   warps 2-5: the epilogue, each reading its quarter of the 128 TMEM lanes
+//   warps 2-5 (2-9 with EXACT): the epilogue, each reading its quarter of the 128 TMEM lanes
 //     (pixels), adding the bias, and storing BF16 after ReLU (or FP32 channel 0).
 // All waits are bounded; on expiry the CTA sets the status word and drains.
 #include <cuda_runtime.h>
@@ -43,7 +43,10 @@ constexpr int W = 128, WP = W + 2;
 constexpr int ROWS = 16;                       // output rows per CTA
 constexpr int NSLOT = 6;                       // staged input rows
 constexpr int CH_BYTES = WP * 16;              // one padded row of one chunk: 2080 B
-constexpr int THREADS = 192;
+// Epilogue warps: one per quarter of the pixels, or two when boundary cases are
+// looked for (each then has half of the output channels).
+constexpr int epi_warps(bool exact) { return exact ? 8 : 4; }
+constexpr int threads(bool exact) { return 64 + 32 * epi_warps(exact); }
 constexpr int QCAP = 64;                       // boundary cases an epilogue warp collects before it recomputes 32
 
 // Shape of one layer: NCI input chunks in global memory, KCH staged chunks
@@ -54,7 +57,7 @@ struct ConvShape {
     static constexpr int ROW_BYTES = KCH * CH_BYTES;
     static constexpr int TAP_BYTES = KCH * NCO * 16;
     static constexpr int WT_BYTES = 9 * TAP_BYTES;
-    static constexpr size_t SMEM = (size_t)WT_BYTES + (size_t)NSLOT * ROW_BYTES + 256 + 4 * QCAP * sizeof(unsigned short);
+    static constexpr size_t SMEM = (size_t)WT_BYTES + (size_t)NSLOT * ROW_BYTES + 256 + 8 * QCAP * sizeof(unsigned short);
     // kind::f16, FP32 accumulate, A = B = BF16, both K-major, N = NCO, M = 128.
     static constexpr unsigned IDESC = ptx::umma_idesc(false, 128, NCO);
 };
@@ -63,6 +66,14 @@ __device__ __forceinline__ unsigned pack2(float a, float b)
 {
     unsigned r;
     asm("cvt.rn.bf16x2.f32 %0, %2, %1;\n" : "=r"(r) : "f"(a), "f"(b));
+    return r;
+}
+
+// Two values to packed BF16 with the ReLU; a NaN gives +0, as fmaxf(v, 0) does.
+__device__ __forceinline__ unsigned pack2_relu(float a, float b)
+{
+    unsigned r;
+    asm("max.bf16x2 %0, %1, %2;\n" : "=r"(r) : "r"(pack2(a, b)), "r"(0u));
     return r;
 }
 
@@ -117,17 +128,18 @@ __device__ float conv_chain(const uint4 *__restrict__ in, size_t plane, const ui
 // epilogue warp collects them over its rows and recomputes 32 at a time, one
 // per lane: recomputing each row's few at once left most lanes idle (32 -> 32
 // layer, 16 frames of 512 x 128: 107 us forward and 185 us backward, against 59
-// and 78 us; 36 us without EXACT). The window is CHAIN_TOL times the pixel's largest sum: the chain of up to 288
+// and 78 us, with packed checks 53 and 66; 36 us without EXACT). The window is CHAIN_TOL times the pixel's largest sum: the chain of up to 288
 // roundings and the tensor core's 18 steps differ by about 1.5e-7 of it (one
 // standard deviation), a sixth of the window.
 constexpr float CHAIN_TOL = 9.5367431640625e-7f;   // 2^-20
 
 template <int NCI, int NCO, int EPI, bool EXACT>
-__global__ void __launch_bounds__(THREADS)
+__global__ void __launch_bounds__(threads(EXACT), EXACT ? 2 : 1)
 conv_tc_kernel(const uint4 *__restrict__ in, const uint4 *__restrict__ wt, const float *__restrict__ bias,
                const uint4 *__restrict__ mask, void *__restrict__ out, int H, int *__restrict__ status)
 {
     using CS = ConvShape<NCI, NCO>;
+    constexpr int THREADS = threads(EXACT), EPW = epi_warps(EXACT), NO = 128 / EPW;   // output channels per epilogue thread
     constexpr int KCH = CS::KCH, ROW_BYTES = CS::ROW_BYTES, WT_BYTES = CS::WT_BYTES;
     extern __shared__ __align__(1024) uint8_t sm[];
     uint8_t *sW = sm;                                  // [9][KCH][NCO][8] BF16
@@ -161,7 +173,7 @@ conv_tc_kernel(const uint4 *__restrict__ in, const uint4 *__restrict__ wt, const
         }
         for (int t = 0; t < 2; ++t) {
             mbar_init(&afull[t], 1);
-            mbar_init(&aempty[t], 4);
+            mbar_init(&aempty[t], EPW);
         }
         mbar_init(wbar, 1);
         mbar_init(dbar, 1);
@@ -262,10 +274,11 @@ conv_tc_kernel(const uint4 *__restrict__ in, const uint4 *__restrict__ wt, const
         // ---------------- epilogue: TMEM -> bias + ReLU, or the mask -> BF16 ----------------
         const int quarter = warp & 3;
         const int j = 32 * quarter + lane;   // pixel = TMEM lane
-        constexpr int NB = EPI == TC_F32 ? 1 : EPI == TC_RELU ? 32 : 0;
+        const int o0 = NO * ((warp - 2) >> 2);   // first output channel
+        constexpr int NB = EPI == TC_F32 ? 1 : EPI == TC_RELU ? NO : 0;
         float b[NB ? NB : 1];
 #pragma unroll
-        for (int o = 0; o < NB; ++o) b[o] = bias[o];
+        for (int o = 0; o < NB; ++o) b[o] = bias[o0 + o];
         unsigned short *queue = reinterpret_cast<unsigned short *>(sRow + NSLOT * ROW_BYTES + 256) + (warp - 2) * QCAP;
         int n_queue = 0;   // entries: row of the strip << 12 | lane << 5 | output channel
         // Entries at .. at + n - 1 (n <= 32), one per lane; the warp has stored these outputs before.
@@ -285,11 +298,11 @@ conv_tc_kernel(const uint4 *__restrict__ in, const uint4 *__restrict__ wt, const
         for (int r = 0; r < nr; ++r) {
             const int t = r & 1;
             // the row's mask is read while its MMAs run
-            const size_t at = ((size_t)f * 4 * HP + r_first + r + 1) * WP + (j + 1);
-            uint4 mk[4];
+            const size_t at = (((size_t)f * 4 + o0 / 8) * HP + r_first + r + 1) * WP + (j + 1);
+            uint4 mk[NO / 8];
             if constexpr (EPI == TC_MASK) {
 #pragma unroll
-                for (int ch = 0; ch < 4; ++ch) mk[ch] = mask[at + (size_t)ch * HP * WP];
+                for (int ch = 0; ch < NO / 8; ++ch) mk[ch] = mask[at + (size_t)ch * HP * WP];
             }
             if (!__all_sync(0xffffffffu, wait(&afull[t], (unsigned)(r >> 1) & 1u))) break;
             tc_fence_after();
@@ -303,51 +316,52 @@ conv_tc_kernel(const uint4 *__restrict__ in, const uint4 *__restrict__ wt, const
                 if (lane == 0) mbar_arrive(&aempty[t]);
                 reinterpret_cast<float *>(out)[((size_t)f * H + r_first + r) * W + j] = __uint_as_float(a0) + b[0];
             } else {
-                unsigned acc[32];
-                tmem_ld32(taddr, acc);
+                float acc[NO];
+#pragma unroll
+                for (int o = 0; o < NO; o += 16) tmem_ld16(taddr + (unsigned)(o0 + o), acc + o);
                 tmem_wait_ld();
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&aempty[t]);
                 uint4 *dst = reinterpret_cast<uint4 *>(out) + at;
-                unsigned redo = 0u;   // bit o: output o is too near a boundary
+                // w[i]: outputs 2 i and 2 i + 1 as packed BF16; d[i]: where the two ends of the window differ
+                unsigned w[NO / 2], d[NO / 2], any = 0u;
+                float tol = 0.0f;
                 if constexpr (EXACT) {
-                    float top = 0.0f;
 #pragma unroll
-                    for (int o = 0; o < 32; ++o) top = fmaxf(top, fabsf(__uint_as_float(acc[o])));
-                    const float tol = CHAIN_TOL * top;
-#pragma unroll
-                    for (int o = 0; o < 32; ++o) {
-                        float v = __uint_as_float(acc[o]);
-                        if constexpr (EPI == TC_RELU) v += b[o];
-                        float up = v + tol, dn = v - tol;
-                        if constexpr (EPI == TC_RELU) {
-                            up = fmaxf(up, 0.0f);
-                            dn = fmaxf(dn, 0.0f);
-                        }
-                        const unsigned pk = pack2(up, dn);
-                        bool near = (pk >> 16) != (pk & 0xFFFFu);
-                        if constexpr (EPI == TC_MASK) {   // masked outputs are zero either way
-                            const uint4 q = mk[o >> 3];
-                            const unsigned w = (o & 7) < 2 ? q.x : (o & 7) < 4 ? q.y : (o & 7) < 6 ? q.z : q.w;
-                            near = near && masked2((o & 1) ? 0xFFFF0000u : 0xFFFFu, w) != 0u;
-                        }
-                        if (near) redo |= 1u << o;
-                    }
+                    for (int o = 0; o < NO; ++o) tol = fmaxf(tol, fabsf(acc[o]));
+                    tol *= CHAIN_TOL;
                 }
 #pragma unroll
-                for (int ch = 0; ch < 4; ++ch) {
-                    float y[8];
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        y[k] = __uint_as_float(acc[ch * 8 + k]);
-                        if constexpr (EPI == TC_RELU) y[k] = fmaxf(y[k] + b[ch * 8 + k], 0.0f);
+                for (int i = 0; i < NO / 2; ++i) {
+                    float2 v = make_float2(acc[2 * i], acc[2 * i + 1]);
+                    if constexpr (EPI == TC_RELU) v = __fadd2_rn(v, make_float2(b[2 * i], b[2 * i + 1]));
+                    w[i] = EPI == TC_RELU ? pack2_relu(v.x, v.y) : pack2(v.x, v.y);
+                    if constexpr (EXACT) {
+                        const float2 up = __fadd2_rn(v, make_float2(tol, tol)), dn = __fadd2_rn(v, make_float2(-tol, -tol));
+                        d[i] = EPI == TC_RELU ? pack2_relu(up.x, up.y) ^ pack2_relu(dn.x, dn.y)
+                                              : pack2(up.x, up.y) ^ pack2(dn.x, dn.y);
                     }
-                    uint4 v = make_uint4(pack2(y[0], y[1]), pack2(y[2], y[3]), pack2(y[4], y[5]), pack2(y[6], y[7]));
-                    if constexpr (EPI == TC_MASK)
-                        v = make_uint4(masked2(v.x, mk[ch].x), masked2(v.y, mk[ch].y), masked2(v.z, mk[ch].z),
-                                       masked2(v.w, mk[ch].w));
-                    dst[(size_t)ch * HP * WP] = v;
+                    if constexpr (EPI == TC_MASK) {   // masked outputs are zero either way
+                        const uint4 q = mk[i >> 2];
+                        const unsigned m = (i & 3) == 0 ? q.x : (i & 3) == 1 ? q.y : (i & 3) == 2 ? q.z : q.w;
+                        w[i] = masked2(w[i], m);
+                        if constexpr (EXACT) d[i] = masked2(d[i], m);
+                    }
+                    if constexpr (EXACT) any |= d[i];
+                }
+#pragma unroll
+                for (int ch = 0; ch < NO / 8; ++ch)
+                    dst[(size_t)ch * HP * WP] = make_uint4(w[4 * ch], w[4 * ch + 1], w[4 * ch + 2], w[4 * ch + 3]);
+                unsigned redo = 0u;   // bit o: output o is too near a boundary
+                if constexpr (EXACT) {
+                    if (any != 0u) {
+#pragma unroll
+                        for (int i = 0; i < NO / 2; ++i) {
+                            if (d[i] & 0xFFFFu) redo |= 1u << (2 * i);
+                            if (d[i] >> 16) redo |= 1u << (2 * i + 1);
+                        }
+                    }
                 }
                 if constexpr (EXACT) {
                     while (true) {
@@ -355,7 +369,7 @@ conv_tc_kernel(const uint4 *__restrict__ in, const uint4 *__restrict__ wt, const
                         if (have == 0u) break;
                         if (redo != 0u) {
                             queue[n_queue + __popc(have & ((1u << lane) - 1u))] =
-                                (unsigned short)(r << 12 | lane << 5 | (__ffs(redo) - 1));
+                                (unsigned short)(r << 12 | lane << 5 | (o0 + __ffs(redo) - 1));
                             redo &= redo - 1u;
                         }
                         n_queue += __popc(have);
@@ -392,7 +406,7 @@ cudaError_t launch_tc(const uint4 *in, const uint4 *wt, const float *bias, const
                       int *status, cudaStream_t st)
 {
     dim3 grid((H + ROWS - 1) / ROWS, F);
-    conv_tc_kernel<NCI, NCO, EPI, EXACT><<<grid, THREADS, ConvShape<NCI, NCO>::SMEM, st>>>(in, wt, bias, mask, out, H,
+    conv_tc_kernel<NCI, NCO, EPI, EXACT><<<grid, threads(EXACT), ConvShape<NCI, NCO>::SMEM, st>>>(in, wt, bias, mask, out, H,
                                                                                            status);
     return cudaGetLastError();
 }
