@@ -220,7 +220,7 @@ features_kernel(const float *__restrict__ bands, const float *__restrict__ E, co
 // One block = 128 pixels of PR output rows; thread = one pixel column, PR x COUT
 // FP32 accumulators. Inputs staged channel-major in shared memory (BF16),
 // weights as FP32 [CIN][9][COUT] (read as broadcast float4).
-enum { EPI_RELU = 0, EPI_MASK = 1, EPI_F32 = 2 };
+enum { EPI_RELU = 0, EPI_MASK = 1 };
 
 template <int NCI, int NCO>
 constexpr size_t conv_cc_smem()
@@ -275,25 +275,16 @@ conv_cc_kernel(const uint4 *__restrict__ in, const float *__restrict__ wt, const
         for (int t = 0; t < 9; ++t) {
             const int u = t / 3, v = t % 3;
             const float *wr = sW + ((size_t)ci * 9 + t) * NCO;
-            if constexpr (NCO % 4 == 0) {
 #pragma unroll
-                for (int o4 = 0; o4 < NCO / 4; ++o4) {
-                    const float4 w4 = reinterpret_cast<const float4 *>(wr)[o4];
+            for (int o4 = 0; o4 < NCO / 4; ++o4) {
+                const float4 w4 = reinterpret_cast<const float4 *>(wr)[o4];
 #pragma unroll
-                    for (int pr = 0; pr < PR; ++pr) {
-                        const float x = xs[pr + u][v];
-                        acc[pr][4 * o4 + 0] = fmaf(x, w4.x, acc[pr][4 * o4 + 0]);
-                        acc[pr][4 * o4 + 1] = fmaf(x, w4.y, acc[pr][4 * o4 + 1]);
-                        acc[pr][4 * o4 + 2] = fmaf(x, w4.z, acc[pr][4 * o4 + 2]);
-                        acc[pr][4 * o4 + 3] = fmaf(x, w4.w, acc[pr][4 * o4 + 3]);
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int o = 0; o < NCO; ++o) {
-                    const float w1 = wr[o];
-#pragma unroll
-                    for (int pr = 0; pr < PR; ++pr) acc[pr][o] = fmaf(xs[pr + u][v], w1, acc[pr][o]);
+                for (int pr = 0; pr < PR; ++pr) {
+                    const float x = xs[pr + u][v];
+                    acc[pr][4 * o4 + 0] = fmaf(x, w4.x, acc[pr][4 * o4 + 0]);
+                    acc[pr][4 * o4 + 1] = fmaf(x, w4.y, acc[pr][4 * o4 + 1]);
+                    acc[pr][4 * o4 + 2] = fmaf(x, w4.z, acc[pr][4 * o4 + 2]);
+                    acc[pr][4 * o4 + 3] = fmaf(x, w4.w, acc[pr][4 * o4 + 3]);
                 }
             }
         }
@@ -305,32 +296,28 @@ conv_cc_kernel(const uint4 *__restrict__ in, const float *__restrict__ wt, const
     for (int pr = 0; pr < PR; ++pr) {
         const int i = r0 + pr;
         if (i >= H) break;
-        if constexpr (EPI == EPI_F32) {
-            reinterpret_cast<float *>(out)[((size_t)f * H + i) * W + j] = acc[pr][0] + bias[0];
-        } else {
-            constexpr int NCH = NCO / 8;
+        constexpr int NCH = NCO / 8;
 #pragma unroll
-            for (int ch = 0; ch < NCH; ++ch) {
-                const size_t o = (((size_t)f * NCH + ch) * HP + (i + 1)) * WP + (j + 1);
-                float y[8];
+        for (int ch = 0; ch < NCH; ++ch) {
+            const size_t o = (((size_t)f * NCH + ch) * HP + (i + 1)) * WP + (j + 1);
+            float y[8];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) y[k] = acc[pr][ch * 8 + k];
-                if constexpr (EPI == EPI_RELU) {
+            for (int k = 0; k < 8; ++k) y[k] = acc[pr][ch * 8 + k];
+            if constexpr (EPI == EPI_RELU) {
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) y[k] = fmaxf(y[k] + bias[ch * 8 + k], 0.0f);
-                } else {
-                    // dX = conv * (act > 0); act is a BF16 ReLU output, so > 0 <=> sign clear and nonzero
-                    const uint4 mk = mask[o];
-                    const unsigned mw[4] = {mk.x, mk.y, mk.z, mk.w};
+                for (int k = 0; k < 8; ++k) y[k] = fmaxf(y[k] + bias[ch * 8 + k], 0.0f);
+            } else {
+                // dX = conv * (act > 0); act is a BF16 ReLU output, so > 0 <=> sign clear and nonzero
+                const uint4 mk = mask[o];
+                const unsigned mw[4] = {mk.x, mk.y, mk.z, mk.w};
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const unsigned h = (k & 1) ? (mw[k >> 1] >> 16) : (mw[k >> 1] & 0xFFFFu);
-                        if (h == 0u || (h & 0x8000u)) y[k] = 0.0f;
-                    }
+                for (int k = 0; k < 8; ++k) {
+                    const unsigned h = (k & 1) ? (mw[k >> 1] >> 16) : (mw[k >> 1] & 0xFFFFu);
+                    if (h == 0u || (h & 0x8000u)) y[k] = 0.0f;
                 }
-                reinterpret_cast<uint4 *>(out)[o] =
-                    make_uint4(pack_bf2(y[0], y[1]), pack_bf2(y[2], y[3]), pack_bf2(y[4], y[5]), pack_bf2(y[6], y[7]));
             }
+            reinterpret_cast<uint4 *>(out)[o] =
+                make_uint4(pack_bf2(y[0], y[1]), pack_bf2(y[2], y[3]), pack_bf2(y[4], y[5]), pack_bf2(y[6], y[7]));
         }
     }
 }
@@ -363,6 +350,63 @@ __global__ void __launch_bounds__(32 * RED_Y) wgrad_reduce_kernel(const float *_
         for (int k = 1; k < RED_Y; ++k) s += sh[k][tx];
         grads[i] = s;
     }
+}
+
+// ------------------------------------------- last layer (32 -> 1, fwd) ----
+// z = b + sum_{c,u,v} w[c][u][v] in[c][i+u-1][j+v-1] in FP32, the chain over
+// channels, then taps, of conv_cc_kernel. One output channel reuses an input 9
+// times only, so the layer is bound by reading its input: a thread takes ZR rows
+// of a pixel column and reads each input row's three pixels of a chunk as 16-byte
+// loads straight from memory (a warp's row of 512 bytes; the shifted re-reads hit
+// L1). Staging channel-major through shared memory took 69 us at 16 frames of
+// 512 x 128; this takes 27.
+constexpr int ZR = 4;
+__global__ void __launch_bounds__(CT)
+conv_last_kernel(const uint4 *__restrict__ in, const float *__restrict__ wt, const float *__restrict__ bias,
+                 float *__restrict__ z, int H, int W)
+{
+    __shared__ __align__(16) float sW[32 * 12];   // [c][9 taps, padded to 12]
+    for (int i = threadIdx.x; i < 32 * 9; i += CT) sW[i / 9 * 12 + i % 9] = wt[i];
+    __syncthreads();
+    const int j = threadIdx.x, r0 = blockIdx.x * ZR, f = blockIdx.y;
+    const int HP = H + 2, WP = W + 2;
+    if (j >= W) return;
+    float acc[ZR];
+#pragma unroll
+    for (int r = 0; r < ZR; ++r) acc[r] = 0.0f;
+#pragma unroll 1
+    for (int c = 0; c < 4; ++c) {
+        uint4 x[ZR + 2][3];
+#pragma unroll
+        for (int k = 0; k < ZR + 2; ++k) {
+            const int row = min(r0 + k, HP - 1);   // rows past the frame feed outputs that are not stored
+            const uint4 *p = in + (((size_t)f * 4 + c) * HP + row) * WP + j;
+#pragma unroll
+            for (int v = 0; v < 3; ++v) x[k][v] = p[v];
+        }
+#pragma unroll
+        for (int k8 = 0; k8 < 8; ++k8) {
+            const float4 *w4 = reinterpret_cast<const float4 *>(sW + (8 * c + k8) * 12);
+            const float4 wa = w4[0], wb = w4[1], wc = w4[2];
+            const float w[9] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w, wc.x};
+            float xs[ZR + 2][3];
+#pragma unroll
+            for (int k = 0; k < ZR + 2; ++k)
+#pragma unroll
+                for (int v = 0; v < 3; ++v) {
+                    const uint4 q = x[k][v];
+                    const unsigned u = k8 < 2 ? q.x : k8 < 4 ? q.y : k8 < 6 ? q.z : q.w;
+                    xs[k][v] = (k8 & 1) ? bf_hi(u) : bf_lo(u);
+                }
+#pragma unroll
+            for (int t = 0; t < 9; ++t)
+#pragma unroll
+                for (int r = 0; r < ZR; ++r) acc[r] = fmaf(xs[r + t / 3][t % 3], w[t], acc[r]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < ZR; ++r)
+        if (r0 + r < H) z[((size_t)f * H + r0 + r) * W + j] = acc[r] + bias[0];
 }
 
 // ------------------------------------------------------------ head ----
@@ -586,7 +630,6 @@ cudaError_t prepare_learn_kernels()
     cudaError_t e;
     if ((e = set_conv_smem<1, 32, EPI_RELU>()) != cudaSuccess) return e;
     if ((e = set_conv_smem<4, 32, EPI_RELU>()) != cudaSuccess) return e;
-    if ((e = set_conv_smem<4, 1, EPI_F32>()) != cudaSuccess) return e;
     if ((e = set_conv_smem<1, 32, EPI_MASK>()) != cudaSuccess) return e;
     if ((e = set_conv_smem<4, 32, EPI_MASK>()) != cudaSuccess) return e;
     return prepare_wgrad();
@@ -759,7 +802,7 @@ cudaError_t run_forward(pam_learn_s *l, const uint4 *feat, int n, bool keep, cud
         const uint4 *in = k ? a[k - 1] : feat;
         // Without pam_learn_configure's tensor cores the activations are the
         // CUDA-core kernel's bits; at nx = 128 tcgen05 makes the same bits faster
-        // (32 -> 32 layer, 16 frames of 512 x 128: 59 us against 467 us).
+        // (32 -> 32 layer, 16 frames of 512 x 128: 53 us against 467 us).
         if (W == 128)
             e = pam::launch_conv_tc_exact(k, in, reinterpret_cast<const uint4 *>(l->prep.wtc[k]), l->prep.bias[k], a[k],
                                           n, H, l->plan->w.status, st);
@@ -769,9 +812,10 @@ cudaError_t run_forward(pam_learn_s *l, const uint4 *feat, int n, bool keep, cud
             e = pam::conv_cc<4, 32, pam::EPI_RELU>(in, l->prep.wf[k], l->prep.bias[k], nullptr, a[k], n, H, W, st);
         if (e != cudaSuccess) return e;
     }
-    e = pam::conv_cc<4, 1, pam::EPI_F32>(a[3], l->prep.wf[4], l->prep.bias[4], nullptr, l->z, n, H, W, st);
+    pam::conv_last_kernel<<<dim3((H + pam::ZR - 1) / pam::ZR, n), pam::CT, 0, st>>>(a[3], l->prep.wf[4], l->prep.bias[4],
+                                                                                    l->z, H, W);
     l->kernels += 5;
-    return e;
+    return cudaGetLastError();
 }
 
 // Loss and gradients of n frames into l->grads (forward included).
