@@ -25,70 +25,66 @@ namespace {
 struct DftFrame {
     size_t rf_off;   // floats: start of the frame's [ne][nt] block
     size_t tw_off;   // float2: start of the frame's twiddle table
+    int f;           // the frame (grid rows take the longest frames first)
     int nt;
     int n_bins;      // bins of this frame (<= the batch's n_bins; the rest of its S rows are zeroed)
 };
 
-constexpr int DFT_WARPS = 8;
+constexpr int DFT_WARPS = 4;
 constexpr int DFT_THREADS = 32 * DFT_WARPS;
-constexpr int DFT_BPW = 4;                      // bins per warp
+constexpr int DFT_BPW = 8;                      // bins per warp
 constexpr int DFT_BINS = DFT_WARPS * DFT_BPW;   // bins per CTA
 constexpr int DFT_T = 64;                       // samples per staged tile
 constexpr int DFT_MAX_NT = 16384;
 
 // S[f][b][e] = sum_t rf[e][t] exp(-2 pi i k_b t / nt)   (Eq. 1, selected bins)
-// by direct summation with the exact index reduction m = k t mod nt into the
-// frame's twiddle table exp(-2 pi i m / nt) (built in FP64). One CTA per
-// (32 bins, frame): warp w owns bins 4w..4w+3, lane l channels l + 32 c,
-// c < CPL. Per 64-sample tile the CTA stages the channels' samples (rows of
-// 64 + 4 floats) and the 32 bins' twiddles for those samples (rows of 64 + 4
-// float2, gathered from the table, which stays in L1/L2, with the index
-// stepped by k per sample), with cp.async into two buffers: tile i+1 is in
-// flight while tile i is summed. Two CTAs share an SM.
-// The inner loop then reads 4 samples of a channel and 4 twiddles of a bin as
-// 16-byte loads (twiddle reads are warp-uniform broadcasts) and updates Re
-// and Im with one packed FMA (fma.rn.f32x2). The sum of each tile is formed on
+// by direct summation, for any nt. With t = t0 + r over tiles of 64 samples,
+//   S = sum_t0 W(k t0) sum_r rf[t0 + r] W(k r),  W(m) = exp(-2 pi i m / nt):
+// the inner twiddles are the same for every tile, so a CTA stages 32 bins x 64
+// of them once, and a tile's sum is turned by one W(k t0) per bin (indices
+// reduced exactly, k t mod nt, into the frame's FP64-built table). Staging a
+// tile's own twiddles instead cost a gather of 8 bytes per (bin, sample) and
+// tile, which with half the bins per warp held the FMA pipe at 45%.
+// One CTA per (32 bins, frame): warp w owns bins 8w..8w+7, lane l channels
+// l + 32 c, c < CPL. The channels' samples (rows of 64 + 4 floats) go through
+// two buffers by cp.async: tile i+1 is in flight while tile i is summed. Two
+// CTAs share an SM.
+// The inner loop reads 4 samples of a channel and 4 twiddles of a bin as 16-byte
+// loads (twiddle reads are warp-uniform broadcasts) and updates Re and Im with
+// one packed FMA (fma.rn.f32x2): 128 of them for 20 loads of 32 wavefronts at 128
+// channels, so the FMA pipe is the bound. The sum of each tile is formed on
 // its own and then added to the total, so the rounding error grows like
 // 64 + nt/64 ulp rather than nt ulp.
+// Measured (GB300, 64 frames of 128 channels, 1024-8192 samples, 300 bins):
+// 1.24 ms against 2.27 ms (FMA pipe 65% busy, two warps per scheduler).
 constexpr int XROW = DFT_T + 4;     // floats per staged channel row
-constexpr int WROW = DFT_T + 4;     // float2 per staged twiddle row
+constexpr int WROW = DFT_T + 2;     // float2 per staged twiddle row (16-byte rows)
 
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-// 4- and 8-byte asynchronous copies global -> shared (cp.async); `valid` false
-// writes zeros without reading.
+// 4-byte asynchronous copy global -> shared (cp.async); `valid` false writes
+// zeros without reading.
 __device__ __forceinline__ void cp_async4(void *dst, const void *src, bool valid)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(smem_addr(dst)), "l"(src),
                  "r"(valid ? 4 : 0)
                  : "memory");
 }
-__device__ __forceinline__ void cp_async8(void *dst, const void *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
 template <int CPL>
-__global__ void __launch_bounds__(DFT_THREADS, CPL >= 8 ? 1 : 2)
+__global__ void __launch_bounds__(DFT_THREADS, 2)
 time_dft_kernel(const float *__restrict__ rf, const DftFrame *__restrict__ frames, const int *__restrict__ bins,
                 int n_bins, int ne, const float2 *__restrict__ tw_all, float2 *__restrict__ S)
 {
     extern __shared__ __align__(16) float2 dsm[];
-    constexpr int WBUF = DFT_BINS * WROW;               // float2 per twiddle buffer
     constexpr int XBUF = 32 * CPL * XROW;               // floats per sample buffer
-    const int f = blockIdx.y;
-    const DftFrame fr = frames[f];
-    const int nt = fr.nt;
-    float2 *wt = dsm;                                                  // [2][DFT_BINS][WROW]
-    float *xs = reinterpret_cast<float *>(wt + 2 * WBUF);             // [2][32 CPL][XROW]
+    const DftFrame fr = frames[blockIdx.y];
+    const int f = fr.f, nt = fr.nt;
+    float2 *wt = dsm;                                                  // [DFT_BINS][WROW] W(k r)
+    float *xs = reinterpret_cast<float *>(wt + DFT_BINS * WROW);       // [2][32 CPL][XROW]
     const float2 *tw = tw_all + fr.tw_off;                             // [nt]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // twiddle staging role: bin bb of the CTA, samples s + 8 j of each tile
-    const int bb = tid >> 3, sg = tid & 7;
-    const int bglob = blockIdx.x * DFT_BINS + bb;
-    const int kb = bglob < fr.n_bins ? bins[(size_t)f * n_bins + bglob] : 0;
-    const int kstep8 = (int)((8LL * kb) % nt);
     const float *x = rf + fr.rf_off;
     // Copies of tile t0 into buffer `buf` (all threads; one commit group).
     auto stage = [&](int t0, int buf) {
@@ -97,47 +93,54 @@ time_dft_kernel(const float *__restrict__ rf, const DftFrame *__restrict__ frame
         for (int e = warp; e < 32 * CPL; e += DFT_WARPS) {
             const bool erow = e < ne;
             const float *row = x + (size_t)(erow ? e : 0) * nt + t0;
+#pragma unroll
             for (int t = lane; t < DFT_T; t += 32)
                 cp_async4(xb + e * XROW + t, row + (t < tn ? t : 0), erow && t < tn);
         }
-        float2 *wb = wt + buf * WBUF + bb * WROW;
-        int idx = (int)(((long long)kb * (t0 + sg)) % nt);
-#pragma unroll
-        for (int j = 0; j < DFT_T / 8; ++j) {
-            cp_async8(wb + sg + 8 * j, tw + idx);
-            idx += kstep8;
-            if (idx >= nt) idx -= nt;
-        }
         cp_async_commit();
     };
+    stage(0, 0);
+    for (int i = tid; i < DFT_BINS * DFT_T; i += DFT_THREADS) {
+        const int bb = i / DFT_T, r = i % DFT_T, bg = blockIdx.x * DFT_BINS + bb;
+        const int k = bg < fr.n_bins ? bins[(size_t)f * n_bins + bg] : 0;
+        wt[bb * WROW + r] = tw[(int)(((long long)k * r) % nt)];
+    }
+    // lane i of each 8 turns bin 8 warp + i of the warp: W(k t0), the index stepped by 64 k per tile
+    const int b0 = blockIdx.x * DFT_BINS + warp * DFT_BPW;
+    const int bt = b0 + (lane & (DFT_BPW - 1));
+    const int kt = bt < fr.n_bins ? bins[(size_t)f * n_bins + bt] : 0;
+    const int kstep = (int)((long long)kt * DFT_T % nt);
+    int tidx = 0;
     float2 tot[DFT_BPW][CPL];
 #pragma unroll
     for (int i = 0; i < DFT_BPW; ++i)
 #pragma unroll
         for (int c = 0; c < CPL; ++c) tot[i][c] = make_float2(0.f, 0.f);
     const int ntiles = (nt + DFT_T - 1) / DFT_T;
-    stage(0, 0);
     for (int it = 0; it < ntiles; ++it) {
         const int buf = it & 1, t0 = it * DFT_T, tn = min(DFT_T, nt - t0);
         if (it + 1 < ntiles) stage(t0 + DFT_T, buf ^ 1);
         else cp_async_commit();                 // empty group keeps the wait count uniform
+        const float2 turn = tw[tidx];           // used after the tile's sum
+        tidx += kstep;
+        if (tidx >= nt) tidx -= nt;
         cp_async_wait1();                       // this thread's copies of tile `it` have landed
-        __syncthreads();                        // ... and everyone else's
+        __syncthreads();                        // ... and everyone else's (and the twiddles)
         const float *xb = xs + buf * XBUF;
-        const float2 *wb = wt + buf * WBUF;
         float2 part[DFT_BPW][CPL];
 #pragma unroll
         for (int i = 0; i < DFT_BPW; ++i)
 #pragma unroll
             for (int c = 0; c < CPL; ++c) part[i][c] = make_float2(0.f, 0.f);
         // samples past tn are zero in xs, so whole groups of 4 are summed
+#pragma unroll 1
         for (int t = 0; t < tn; t += 4) {
             float4 xv[CPL];
 #pragma unroll
             for (int c = 0; c < CPL; ++c) xv[c] = *reinterpret_cast<const float4 *>(xb + (lane + 32 * c) * XROW + t);
 #pragma unroll
             for (int i = 0; i < DFT_BPW; ++i) {
-                const float4 *wp = reinterpret_cast<const float4 *>(wb + (warp * DFT_BPW + i) * WROW + t);
+                const float4 *wp = reinterpret_cast<const float4 *>(wt + (warp * DFT_BPW + i) * WROW + t);
                 const float4 w01 = wp[0], w23 = wp[1];
                 const float2 w0 = make_float2(w01.x, w01.y), w1 = make_float2(w01.z, w01.w);
                 const float2 w2 = make_float2(w23.x, w23.y), w3 = make_float2(w23.z, w23.w);
@@ -153,12 +156,17 @@ time_dft_kernel(const float *__restrict__ rf, const DftFrame *__restrict__ frame
             }
         }
 #pragma unroll
-        for (int i = 0; i < DFT_BPW; ++i)
+        for (int i = 0; i < DFT_BPW; ++i) {
+            const float wr = __shfl_sync(0xffffffffu, turn.x, i), wi = __shfl_sync(0xffffffffu, turn.y, i);
 #pragma unroll
-            for (int c = 0; c < CPL; ++c) tot[i][c] = __fadd2_rn(tot[i][c], part[i][c]);
+            for (int c = 0; c < CPL; ++c) {
+                const float2 p = part[i][c];
+                tot[i][c] = __ffma2_rn(make_float2(p.x, p.x), make_float2(wr, wi),
+                                       __ffma2_rn(make_float2(p.y, p.y), make_float2(-wi, wr), tot[i][c]));
+            }
+        }
         __syncthreads();                        // buffer `buf` is free for tile it + 2
     }
-    const int b0 = blockIdx.x * DFT_BINS + warp * DFT_BPW;
 #pragma unroll
     for (int i = 0; i < DFT_BPW; ++i) {
         if (b0 + i >= n_bins) continue;
@@ -171,46 +179,43 @@ time_dft_kernel(const float *__restrict__ rf, const DftFrame *__restrict__ frame
     }
 }
 
-size_t dft_smem(int, int cpl)
+size_t dft_smem(int cpl)
 {
-    return 2 * ((size_t)DFT_BINS * WROW * sizeof(float2) + (size_t)32 * cpl * XROW * sizeof(float));
+    return (size_t)DFT_BINS * WROW * sizeof(float2) + 2 * (size_t)32 * cpl * XROW * sizeof(float);
 }
 
 template <int CPL>
 cudaError_t launch_dft_t(const float *rf, const DftFrame *frames, const int *bins, int n_bins, int ne, int F,
-                         const float2 *tw, float2 *S, int max_nt, cudaStream_t st)
+                         const float2 *tw, float2 *S, cudaStream_t st)
 {
     dim3 grid((unsigned)((n_bins + DFT_BINS - 1) / DFT_BINS), (unsigned)F);
-    time_dft_kernel<CPL><<<grid, DFT_THREADS, dft_smem(max_nt, CPL), st>>>(rf, frames, bins, n_bins, ne, tw, S);
+    time_dft_kernel<CPL><<<grid, DFT_THREADS, dft_smem(CPL), st>>>(rf, frames, bins, n_bins, ne, tw, S);
     return cudaGetLastError();
 }
 
 cudaError_t launch_dft(int cpl, const float *rf, const DftFrame *frames, const int *bins, int n_bins, int ne, int F,
-                       const float2 *tw, float2 *S, int max_nt, cudaStream_t st)
+                       const float2 *tw, float2 *S, cudaStream_t st)
 {
     switch (cpl) {
-    case 1: return launch_dft_t<1>(rf, frames, bins, n_bins, ne, F, tw, S, max_nt, st);
-    case 2: return launch_dft_t<2>(rf, frames, bins, n_bins, ne, F, tw, S, max_nt, st);
-    case 4: return launch_dft_t<4>(rf, frames, bins, n_bins, ne, F, tw, S, max_nt, st);
-    case 8: return launch_dft_t<8>(rf, frames, bins, n_bins, ne, F, tw, S, max_nt, st);
+    case 1: return launch_dft_t<1>(rf, frames, bins, n_bins, ne, F, tw, S, st);
+    case 2: return launch_dft_t<2>(rf, frames, bins, n_bins, ne, F, tw, S, st);
+    case 4: return launch_dft_t<4>(rf, frames, bins, n_bins, ne, F, tw, S, st);
     default: return cudaErrorInvalidValue;
     }
 }
 
+template <int CPL>
+cudaError_t set_dft_smem()
+{
+    return cudaFuncSetAttribute(time_dft_kernel<CPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dft_smem(CPL));
+}
+
 cudaError_t prepare_dft()
 {
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(time_dft_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)dft_smem(DFT_MAX_NT, 1))) != cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(time_dft_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)dft_smem(DFT_MAX_NT, 2))) != cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(time_dft_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)dft_smem(DFT_MAX_NT, 4))) != cudaSuccess)
-        return e;
-    return cudaFuncSetAttribute(time_dft_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)dft_smem(DFT_MAX_NT, 8));
+    cudaError_t e = set_dft_smem<1>();
+    if (e == cudaSuccess) e = set_dft_smem<2>();
+    if (e == cudaSuccess) e = set_dft_smem<4>();
+    return e;
 }
 
 pam_status fail(pam_status s, const std::string &msg) { return set_error(s, msg.c_str()); }
@@ -242,7 +247,7 @@ size_t round4(size_t v) { return (v + 3) & ~(size_t)3; }
 
 struct pam_batch_s {
     pam_plan_s *base = nullptr;     // geometry, apodization, workspace for F frames of n_bins bins
-    int F = 0, n_bins = 0, ne = 0, nx = 0, napq = 0, max_nt = 0, max_npix = 0, cpl = 4;
+    int F = 0, n_bins = 0, ne = 0, nx = 0, napq = 0, max_npix = 0, cpl = 4;
     int grid = 0, grid_override = 0, n_items = 0;
     int rpl = 1;                     // depth rows per lane of the fused kernel (2 for nx >= 64)
     std::vector<int> nt, nz, nbf, bins_h;   // per frame: samples, rows, bin count; bins [F][n_bins]
@@ -319,7 +324,7 @@ pam_status frame_bins(const pam_plan_desc *c, const pam_frame_desc &fd, int n_bi
 pam_status enqueue(pam_batch_s *b, const float *rf, float *image, float *rho_n, cudaStream_t st)
 {
     pam_plan_s &p = *b->base;
-    cudaError_t e = pam::launch_dft(b->cpl, rf, b->dft, b->bins, b->n_bins, b->ne, b->F, b->tw, p.w.S, b->max_nt, st);
+    cudaError_t e = pam::launch_dft(b->cpl, rf, b->dft, b->bins, b->n_bins, b->ne, b->F, b->tw, p.w.S, st);
     if (e != cudaSuccess) return pam::cuda_fail(e, "time DFT launch");
     e = pam::launch_lateral_frames(p, b->F, b->napq, p.t.apod, b->live, (size_t)b->n_bins * b->nx, st);
     if (e != cudaSuccess) return pam::cuda_fail(e, "lateral DFT launch");
@@ -390,7 +395,6 @@ pam_status pam_batch_create(const pam_plan_desc *common, const pam_frame_desc *f
         b->nbf.push_back((int)fb.size());
         fb.resize(b->n_bins, 0);
         b->bins_h.insert(b->bins_h.end(), fb.begin(), fb.end());
-        b->max_nt = std::max(b->max_nt, fd.n_samples);
         max_nz = std::max(max_nz, fd.nz);
     }
     // Base plan: the shared geometry, apodization and workspace. Its own bins
@@ -412,7 +416,7 @@ pam_status pam_batch_create(const pam_plan_desc *common, const pam_frame_desc *f
     pam_plan_s &p = *b->base;
     b->ne = p.ne;
     b->nx = p.nx;
-    b->cpl = b->ne <= 32 ? 1 : b->ne <= 64 ? 2 : b->ne <= 128 ? 4 : 8;
+    b->cpl = b->ne <= 32 ? 1 : b->ne <= 64 ? 2 : 4;   // at most 128 channels (built lateral lengths)
     size_t tw_total = 0;
     std::vector<size_t> tw_off(n_frames);
     for (int f = 0; f < n_frames; ++f) {
@@ -471,6 +475,7 @@ pam_status pam_batch_create(const pam_plan_desc *common, const pam_frame_desc *f
     e = cudaMemcpy(b->bins, b->bins_h.data(), sizeof(int) * FB, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->dft, dh.data(), sizeof(pam::DftFrame) * n_frames, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
+        dh[f].f = f;
         e = cudaMemcpy(b->frames, fh.data(), sizeof(pam::BatchFrame) * n_frames, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->items, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice);
     for (int f = 0; f < n_frames && e == cudaSuccess; ++f)
@@ -485,6 +490,8 @@ pam_status pam_batch_create(const pam_plan_desc *common, const pam_frame_desc *f
         return pam::cuda_fail(e, "batch tables");
     }
     *out = b;
+    // longest frames first, so that the time DFT's last CTAs are short ones
+    std::stable_sort(dh.begin(), dh.end(), [](const pam::DftFrame &u, const pam::DftFrame &v) { return u.nt > v.nt; });
     return PAM_OK;
 }
 
