@@ -321,7 +321,8 @@ pam_status pam_profile_read(pam_plan_t p, double *prop_ms, long long *prop_launc
  * n_samples may be any integer (no power-of-2 requirement). One call runs a
  * fixed sequence of 4 kernels (time DFT, lateral FFT, a persistent
  * propagate-and-correlate kernel over (frame, row tile) work items, and the
- * per-frame normalisation), replayed as a CUDA graph that the batch captures
+ * per-frame normalisation; 5 for few work items, whose bins are divided among
+ * the SMs and added up), replayed as a CUDA graph that the batch captures
  * on its first call and again whenever the buffers change.
  * ------------------------------------------------------------------------ */
 typedef struct pam_batch_s *pam_batch_t;
@@ -371,11 +372,12 @@ pam_status pam_batch_sync(pam_batch_t b, void *stream);
 
 /* Tuning knobs. use_graph 0 launches the kernels directly (no graph);
  * persistent_ctas > 0 sets the grid of the persistent kernel (0: one per SM,
- * the most that fit; at most one per work item). */
+ * the most that fit; at most one per work item; for each chunk of the bins where
+ * few work items have theirs divided). Results do not depend on it. */
 pam_status pam_batch_configure(pam_batch_t b, int use_graph, int persistent_ctas);
 
 /* Work items (frame, row tile), the persistent grid in use, and the libpam
- * kernels launched so far (a graph launch counts its 4 kernels). Any output
+ * kernels launched so far (a graph launch counts its 4 or 5 kernels). Any output
  * pointer may be NULL. */
 pam_status pam_batch_info(pam_batch_t b, int *n_items, int *persistent_ctas, long long *kernel_launches);
 
@@ -426,8 +428,8 @@ pam_status pam_image_metrics(const float *maps, int n_frames, int nz, int nx, do
  * input channel 0), with Adam (Kingma and Ba 2015: beta1 0.9, beta2 0.999,
  * eps 1e-8), all on the GPU.
  *
- * Error gate: per frame, the exact method runs on the tile of 16 depth rows
- * (nx = 128; 2048 / nx rows otherwise) that holds the brightest pixel of the
+ * Error gate: per frame, the exact method runs on the tile of 32 depth rows
+ * (nx = 128; 4096 / nx rows otherwise) that holds the brightest pixel of the
  * predicted image. If the relative L2 distance there between rho_pred^2 E and
  * rho^2 E exceeds gate_tol, the frame is recomputed by the plain AS-TAX path,
  * on the GPU, within the same call.

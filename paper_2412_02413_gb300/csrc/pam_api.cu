@@ -289,6 +289,7 @@ pam_status alloc_plan(pam_plan_s *p)
     const size_t part_floats = std::max(p->w.part_units * (size_t)pam::n_acc(p->n_apod) * npix,
                                         pam::prop_seg_part_floats(*p));
     PAM_TRY(dalloc(&p->w.part, part_floats));
+    p->w.part_floats = part_floats;
     p->seg_ok = true;
     PAM_TRY(dalloc(&p->w.rho_tmp, F * npix));
     PAM_TRY(dalloc(&p->w.e_tmp, F * npix));

@@ -268,10 +268,15 @@ struct pam_batch_s {
     const float *g_rf = nullptr;
     float *g_img = nullptr, *g_rho = nullptr;
     int g_grid = 0;
+    int n_kernels = 0;               // of one call
     long long kernels = 0;
 };
 
 namespace {
+
+// Work units (items times bin chunks) up to which items are split: 150 MB of
+// partial sums at nx = 128, within the workspace of the batches that need it.
+constexpr size_t kMaxUnits = 1024;
 
 void batch_free(pam_batch_s *b)
 {
@@ -340,13 +345,25 @@ pam_status enqueue(pam_batch_s *b, const float *rf, float *image, float *rho_n, 
     out.e_tmp = p.w.e_tmp;
     out.fmax = p.w.fmax;
     out.status = p.w.status;
-    const int grid = b->grid_override > 0 ? std::min(b->grid_override, b->n_items) : b->grid;
-    e = pam::launch_prop_batch(b->nx, b->napq, grid, b->frames, b->items, b->n_items, b->counter, out, st, nullptr,
-                               b->rpl);
+    pam::ItemWork k;
+    k.frames = b->frames;
+    k.items = b->items;
+    k.n_items = b->n_items;
+    k.counter = b->counter;
+    k.sms = p.num_sms;
+    k.part = p.w.part;
+    k.cap = (int)std::min<size_t>(kMaxUnits, p.w.part_floats /
+                                                 ((size_t)pam::n_acc(b->napq) * pam::prop_rows_per_cta(b->nx, b->rpl) * b->nx));
+    // persistent CTAs for each bin chunk of the items, at most one per SM altogether
+    const int units = pam::item_units(k.n_items, k.sms, k.cap), chunks = units / k.n_items;
+    k.grid = std::min(units, b->grid_override > 0 ? b->grid_override * chunks
+                                                  : pam::prop_ctas_per_sm() * p.num_sms);
+    e = pam::launch_prop_batch(b->nx, b->napq, k, out, st, b->rpl);
     if (e != cudaSuccess) return pam::cuda_fail(e, "propagate/correlate launch");
     e = pam::launch_normalize_batch(b->F, b->max_npix, b->frames, out, st);
     if (e != cudaSuccess) return pam::cuda_fail(e, "normalise launch");
-    b->kernels += 4;
+    b->n_kernels = 3 + pam::prop_batch_kernels(k);
+    b->kernels += b->n_kernels;
     return PAM_OK;
 }
 
@@ -458,6 +475,7 @@ pam_status pam_batch_create(const pam_plan_desc *common, const pam_frame_desc *f
     for (int f = 0; f < n_frames; ++f) {
         dh[f].rf_off = b->rf_off[f];
         dh[f].tw_off = tw_off[f];
+        dh[f].f = f;
         dh[f].nt = b->nt[f];
         dh[f].n_bins = b->nbf[f];
         pam::BatchFrame &x = fh[f];
@@ -472,10 +490,11 @@ pam_status pam_batch_create(const pam_plan_desc *common, const pam_frame_desc *f
         x.dzf = (float)p.d.dz_m;
         x.out_off = b->px_off[f];
     }
+    // longest frames first, so that the time DFT's last CTAs are short ones
+    std::stable_sort(dh.begin(), dh.end(), [](const pam::DftFrame &u, const pam::DftFrame &v) { return u.nt > v.nt; });
     e = cudaMemcpy(b->bins, b->bins_h.data(), sizeof(int) * FB, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->dft, dh.data(), sizeof(pam::DftFrame) * n_frames, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
-        dh[f].f = f;
         e = cudaMemcpy(b->frames, fh.data(), sizeof(pam::BatchFrame) * n_frames, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->items, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice);
     for (int f = 0; f < n_frames && e == cudaSuccess; ++f)
@@ -490,8 +509,6 @@ pam_status pam_batch_create(const pam_plan_desc *common, const pam_frame_desc *f
         return pam::cuda_fail(e, "batch tables");
     }
     *out = b;
-    // longest frames first, so that the time DFT's last CTAs are short ones
-    std::stable_sort(dh.begin(), dh.end(), [](const pam::DftFrame &u, const pam::DftFrame &v) { return u.nt > v.nt; });
     return PAM_OK;
 }
 
@@ -565,7 +582,7 @@ pam_status pam_batch_as_tax(pam_batch_t b, const float *rf, float *image, float 
     }
     cudaError_t e = cudaGraphLaunch(b->exec, st);
     if (e != cudaSuccess) return pam::cuda_fail(e, "graph launch");
-    b->kernels += 4;
+    b->kernels += b->n_kernels;
     return PAM_OK;
 }
 

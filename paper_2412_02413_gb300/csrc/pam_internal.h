@@ -59,11 +59,25 @@ struct BatchFrame {
     size_t out_off;         // pixel offset of the frame's maps
 };
 
+// The persistent kernel over (frame, row tile) items (launch_prop_batch).
+struct ItemWork {
+    int grid = 0;                        // CTAs
+    const BatchFrame *frames = nullptr;
+    const int2 *items = nullptr;         // (frame, row tile of prop_rows_per_cta(nx, rpl) rows)
+    int n_items = 0;
+    const int *n_items_dev = nullptr;    // optional: a device int that caps n_items when the kernel starts
+    int *counter = nullptr;              // work-queue head, zero before the launch
+    int sms = 0;                         // SMs the bins of few items are split over
+    float *part = nullptr;               // `cap` slots of n_acc x rows x nx floats for the split items' sums
+    int cap = 0;                         // (fewer than 2: items are not split)
+};
+
 struct Workspace {
     float2 *S = nullptr;        // [max_frames][n_bins][n_elem]      selected time bins
     float2 *Q = nullptr;        // [max_frames][n_bins][napq][nx]    apodized lateral spectra / nx
     float *part = nullptr;      // [units][n_acc][nz][nx]            per-split accumulator partials
     size_t part_units = 0;
+    size_t part_floats = 0;     // size of part
     float *rho_tmp = nullptr;   // [max_frames][nz][nx]              rho before normalisation
     float *e_tmp = nullptr;     // [max_frames][nz][nx]              sum_k |sum_q p_q|^2
     unsigned *fmax = nullptr;   // [max_frames]                      max rho bits per frame
@@ -161,12 +175,13 @@ bool prop_seg_mode(const pam_plan_s &p, int n_split, bool fields);
 int prop_seg_ctas(const pam_plan_s &p, int n_frames);
 size_t prop_seg_part_floats(const pam_plan_s &p);
 // Batch (pam_batch.cu): the persistent propagate-and-correlate kernel over
-// (frame, row tile) items and the per-frame normalisation.
-// n_items_dev (optional): a device int that caps n_items when the kernel starts.
+// (frame, row tile) items, their bins split where the items alone would leave
+// SMs idle (a second kernel then adds the chunks), and the per-frame
+// normalisation.
 // rpl: depth rows per lane; the items' row tiles are prop_rows_per_cta(nx, rpl) rows.
-cudaError_t launch_prop_batch(int nx, int napq, int grid, const BatchFrame *frames, const int2 *items, int n_items,
-                              int *counter, const EpiOut &out, cudaStream_t st, const int *n_items_dev = nullptr,
-                              int rpl = 1);
+cudaError_t launch_prop_batch(int nx, int napq, const ItemWork &k, const EpiOut &out, cudaStream_t st, int rpl);
+int prop_batch_kernels(const ItemWork &k);               // kernels it launches
+int item_units(int n_items, int sms, int cap);           // items times their bin chunks
 // Full-aperture energy split by bins: the fused kernel (one aperture, whatever
 // Q holds) over n_bands contiguous chunks of Omega, chunk b = bins
 // [floor(n_bins b / n_bands), floor(n_bins (b+1) / n_bands)), each chunk's

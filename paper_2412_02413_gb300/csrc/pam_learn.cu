@@ -642,7 +642,9 @@ cudaError_t prepare_learn_kernels()
 struct pam_learn_s {
     pam_plan_s *plan = nullptr;   // owned: geometry, tables, time/lateral workspace
     pam_plan_s *gemm = nullptr;   // owned, with tensor cores on: BF16 form for the band energies
-    int F = 0, H = 0, W = 0, HP = 0, WP = 0, tiles = 0, rpt = 0, n_sms = 0;
+    int F = 0, H = 0, W = 0, HP = 0, WP = 0, n_sms = 0;
+    int rpt = 0, tiles = 0;       // rows of the gate's and the fallback's tiles, tiles per frame
+    int rpl = 1, tiles_x = 0;     // training targets: rows per lane, tiles per frame
     size_t npix = 0, ppix = 0;    // nz*nx, (nz+2)*(nx+2)
     float gate_tol = 0.05f;
     bool use_tc = false;
@@ -866,6 +868,29 @@ cudaError_t run_grads(pam_learn_s *l, const uint4 *feat, const float *target, in
     return cudaSuccess;
 }
 
+// The exact method on `n_items` (frame, row tile) items. With `spread`, the bins
+// of few items are divided among the SMs; without it an item's bins are summed in
+// one pass, the order of the plain path with one split. `head` is the queue head,
+// zeroed by gate_items_kernel.
+cudaError_t run_items(pam_learn_s *l, const int2 *items, int n_items, const int *n_items_dev, int *head, int rpl,
+                      bool spread, const pam::EpiOut &out, cudaStream_t st)
+{
+    pam_plan_s &p = *l->plan;
+    pam::ItemWork k;
+    k.frames = l->frames;
+    k.items = items;
+    k.n_items = n_items;
+    k.n_items_dev = n_items_dev;
+    k.counter = head;
+    k.sms = l->n_sms;
+    k.part = p.w.part;
+    if (spread) k.cap = (int)std::min<size_t>(1024, p.w.part_floats / ((size_t)6 * pam::prop_rows_per_cta(l->W, rpl) * l->W));
+    const int ctas = pam::prop_ctas_per_sm() * l->n_sms;
+    k.grid = n_items_dev ? ctas : std::min(ctas, pam::item_units(n_items, k.sms, k.cap));
+    l->kernels += pam::prop_batch_kernels(k);
+    return pam::launch_prop_batch(l->W, 3, k, out, st, rpl);
+}
+
 pam_status check_frames(pam_learn_s *l, int n)
 {
     if (!l) return lfail(PAM_ERR_INVALID_ARG, "learned-form handle is NULL");
@@ -907,6 +932,9 @@ pam_status pam_learn_create(const pam_plan_desc *d, pam_learn_t *out)
     l->ppix = (size_t)l->HP * l->WP;
     l->rpt = pam::prop_rows_per_cta(l->W);
     l->tiles = (l->H + l->rpt - 1) / l->rpt;
+    // training targets run two rows per lane where that makes larger tiles (as batches do)
+    l->rpl = l->W >= 64 ? 2 : 1;
+    l->tiles_x = (l->H + pam::prop_rows_per_cta(l->W, l->rpl) - 1) / pam::prop_rows_per_cta(l->W, l->rpl);
     l->n_sms = p.num_sms;
     l->loss_blocks = epi_grid(l->npix);
     const size_t F = (size_t)l->F;
@@ -961,14 +989,14 @@ pam_status pam_learn_create(const pam_plan_desc *d, pam_learn_t *out)
     LALLOC(zalloc(&l->peak, F));
     LALLOC(zalloc(&l->frames, F));
     LALLOC(zalloc(&l->items_gate, F));
-    LALLOC(zalloc(&l->items_all, F * l->tiles));
+    LALLOC(zalloc(&l->items_all, F * l->tiles_x));
     LALLOC(zalloc(&l->items_fb, F * l->tiles));
     LALLOC(zalloc(&l->counters, 4));
     LALLOC(zalloc(&l->gate_err, F));
     LALLOC(zalloc(&l->gate_pass, F));
     {
         std::vector<pam::BatchFrame> fr(F);
-        std::vector<int2> all(F * l->tiles);
+        std::vector<int2> all(F * l->tiles_x);
         for (size_t f = 0; f < F; ++f) {
             pam::BatchFrame &b = fr[f];
             b.Q = p.w.Q + f * p.n_bins * pam::q_per_bin(3, p.nx);
@@ -981,7 +1009,7 @@ pam_status pam_learn_create(const pam_plan_desc *d, pam_learn_t *out)
             b.z0f = (float)p.d.z0_m;
             b.dzf = (float)p.d.dz_m;
             b.out_off = f * l->npix;
-            for (int t = 0; t < l->tiles; ++t) all[f * l->tiles + t] = make_int2((int)f, t);
+            for (int t = 0; t < l->tiles_x; ++t) all[f * l->tiles_x + t] = make_int2((int)f, t);
         }
         LALLOC(cudaMemcpy(l->frames, fr.data(), sizeof(pam::BatchFrame) * F, cudaMemcpyHostToDevice));
         LALLOC(cudaMemcpy(l->items_all, all.data(), sizeof(int2) * all.size(), cudaMemcpyHostToDevice));
@@ -1123,10 +1151,8 @@ pam_status pam_learn_example(pam_learn_t l, const float *rf, int n_frames, void 
         out.e_tmp = p.w.e_tmp;
         out.fmax = l->fmax_x;
         out.status = p.w.status;
-        const int n_items = n_frames * l->tiles;
-        LTRY(pam::launch_prop_batch(l->W, 3, std::min(pam::prop_ctas_per_sm() * l->n_sms, n_items), l->frames, l->items_all, n_items,
-                                    l->counters + 1, out, st));
-        l->kernels += 3;
+        LTRY(run_items(l, l->items_all, n_frames * l->tiles_x, nullptr, l->counters + 1, l->rpl, true, out, st));
+        l->kernels += 2;
     }
     LTRY(mark_done(l, st));
     return PAM_OK;
@@ -1227,8 +1253,7 @@ pam_status pam_learn_tax(pam_learn_t l, const float *rf, int n_frames, float *im
         out.e_tmp = p.w.e_tmp;
         out.fmax = l->fmax_g;
         out.status = p.w.status;
-        LTRY(pam::launch_prop_batch(l->W, 3, std::min(pam::prop_ctas_per_sm() * l->n_sms, n), l->frames, l->items_gate, n, l->counters,
-                                    out, st));
+        LTRY(run_items(l, l->items_gate, n, nullptr, l->counters, 1, true, out, st));
         float *gerr = gate_err ? gate_err + f0 : l->gate_err;
         int *gpass = gate_pass ? gate_pass + f0 : l->gate_pass;
         pam::gate_check_kernel<<<n, pam::EPI_THREADS, 0, st>>>(l->items_gate, l->rho, l->E, p.w.rho_tmp, p.w.e_tmp,
@@ -1237,13 +1262,12 @@ pam_status pam_learn_tax(pam_learn_t l, const float *rf, int n_frames, float *im
         LTRY(cudaGetLastError());
         // fallback: the plain method on every row tile of the frames that missed the gate
         out.fmax = l->fmax_x;
-        LTRY(pam::launch_prop_batch(l->W, 3, pam::prop_ctas_per_sm() * l->n_sms, l->frames, l->items_fb, n * l->tiles, l->counters + 1, out,
-                                    st, l->counters + 2));
+        LTRY(run_items(l, l->items_fb, n * l->tiles, l->counters + 2, l->counters + 1, 1, false, out, st));
         pam::learn_finalize_kernel<<<g, pam::EPI_THREADS, 0, st>>>(
             gpass, l->rho, l->rmax, l->E, p.w.rho_tmp, p.w.e_tmp, l->fmax_x, (int)l->npix, image + (size_t)f0 * l->npix,
             rho_n ? rho_n + (size_t)f0 * l->npix : nullptr);
         LTRY(cudaGetLastError());
-        l->kernels += 7;
+        l->kernels += 5;
     }
     LTRY(mark_done(l, st));
     return PAM_OK;

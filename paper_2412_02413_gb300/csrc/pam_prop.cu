@@ -903,17 +903,46 @@ epi_normalize_kernel(const float4 *__restrict__ rho_tmp, const float4 *__restric
     if (rho_n) rho_n[o] = rn;
 }
 
+// Bin chunks per work item of prop_batch_kernel: one where the items fill the
+// SMs, more where a few items (or a last wave of few) would leave most of them
+// idle. The split that minimises waves x (chunk time + the cost of a partial: its
+// sums go to memory and back, about 10 us against 1 ms for an item's 300 bins at
+// nx = 128), at most kMaxItemSplit and what `cap` slots of partial sums hold.
+// It depends on the items and the device alone, not on the grid, so that a
+// launch's grouping of the sums, and with it every bit, does not depend on the
+// grid. Measured (GB300): the gate tiles of 32 frames (32 items of 32 rows x 300
+// bins) 175 us and 26 us for the sums, against 705 us unsplit.
+constexpr int kMaxItemSplit = 48;
+__host__ __device__ __forceinline__ int item_split(int n_items, int sms, int cap)
+{
+    int best = 1, cost = 0x7fffffff;
+    for (int s = 1; s <= kMaxItemSplit; ++s) {
+        if (s > 1 && (long long)n_items * s > cap) break;
+        const int waves = (int)(((long long)n_items * s + sms - 1) / sms);
+        const long long c = (long long)waves * (10000 / s + (s > 1 ? 100 : 0));
+        if (c < cost) {
+            cost = (int)c;
+            best = s;
+        }
+    }
+    return best;
+}
+
 // Persistent form for a batch of frames with their own bins and depth grids
-// (uneven sample counts and depth ranges). Work items are (frame, row tile)
-// pairs taken from a global counter; an item runs every bin of its frame, so
-// its per-pixel epilogue follows directly from the registers. The staging
-// ring's position carries over from item to item.
+// (uneven sample counts and depth ranges). Work units are (frame, row tile)
+// items times the bin chunks of item_split, taken from a global counter. With
+// one chunk a unit runs every bin of its frame and its per-pixel epilogue
+// follows directly from the registers; otherwise unit u writes its sums to
+// part[u][NACC][RPC][NX] and epi_reduce_items_kernel adds an item's chunks in
+// order. The staging ring's position carries over from unit to unit.
 template <int NAP, int NX, int RPL>
 __global__ void __launch_bounds__(32 * prop_warps(RPL, NX), PROP_CTAS)
 prop_batch_kernel(const BatchFrame *__restrict__ frames, const int2 *__restrict__ items, int n_items,
-                  const int *__restrict__ n_items_dev, int *__restrict__ counter, EpiOut out)
+                  const int *__restrict__ n_items_dev, int *__restrict__ counter, int sms, int cap,
+                  float *__restrict__ part, EpiOut out)
 {
     if (n_items_dev) n_items = min(n_items, *n_items_dev);
+    const int split = item_split(n_items, sms, cap);
     using S = Shape<NX, RPL>;
     constexpr int L2 = S::L2, LPR = S::LPR, RPW = S::RPW, RPC = S::RPC, KPL = S::KPL;
     constexpr int NACC = Acc<NAP>::N;
@@ -921,7 +950,7 @@ prop_batch_kernel(const BatchFrame *__restrict__ frames, const int2 *__restrict_
     constexpr int NT = 32 * prop_warps(RPL, NX);
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const PropSmem<NAP, NX, RPL> sm(smem_raw);
-    __shared__ int s_item;
+    __shared__ int s_unit;
     __shared__ float wmax[NT / 32];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int r = lane / LPR, g = (lane % LPR) / L2, n2 = lane % L2;
@@ -929,13 +958,15 @@ prop_batch_kernel(const BatchFrame *__restrict__ frames, const int2 *__restrict_
     const unsigned tcol = acc_tcol(tbase, warp, NACC, RPL);
     unsigned seq = 0;
     for (;;) {
-        if (tid == 0) s_item = atomicAdd(counter, 1);
+        if (tid == 0) s_unit = atomicAdd(counter, 1);
         __syncthreads();
-        const int it = s_item;
+        const int unit = s_unit;
         __syncthreads();
+        const int it = unit / split, ch = unit - it * split;
         if (it >= n_items) break;
         const int2 w = items[it];
         const BatchFrame fr = frames[w.x];
+        const int b0 = (int)((long long)fr.n_bins * ch / split), b1 = (int)((long long)fr.n_bins * (ch + 1) / split);
         int jr[RPL], jj[RPL];
         float zj[RPL];
         bool rok[RPL];
@@ -947,9 +978,9 @@ prop_batch_kernel(const BatchFrame *__restrict__ frames, const int2 *__restrict_
             zj[rr] = fr.z0f + (float)jj[rr] * fr.dzf;
             acc_zero<NAP>(tcol + (unsigned)(rr * 8 * NACC));
         }
-        const bool ok = prop_bins<NAP, NX, false, RPL>(sm, fr.Q, fr.phase, fr.bin_evan, 0, fr.n_bins, jj, zj, seq,
+        const bool ok = prop_bins<NAP, NX, false, RPL>(sm, fr.Q, fr.phase, fr.bin_evan, b0, b1 - b0, jj, zj, seq,
                                                        tcol, nullptr, false, 0);
-        seq += (unsigned)fr.n_bins;
+        seq += (unsigned)(b1 - b0);
         if (!ok && lane == 0) atomicOr(out.status, 1);
         if (__syncthreads_or(!ok)) break;
         float rmax = 0.0f;
@@ -957,18 +988,86 @@ prop_batch_kernel(const BatchFrame *__restrict__ frames, const int2 *__restrict_
         for (int rr = 0; rr < RPL; ++rr) {
             float acc[NOUT][NACC];
             acc_read<NAP>(tcol + (unsigned)(rr * 8 * NACC), acc);   // warp-collective
-            if (rok[rr]) {
+            if (split == 1) {
+                if (rok[rr]) {
+#pragma unroll
+                    for (int o = 0; o < NOUT; ++o) {
+                        const int k1 = n2 * KPL + o / L2, k2 = o % L2;
+                        const int i = 2 * (k1 + 8 * k2) + g;
+                        rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc[o], out, 0, fr.out_off + (size_t)jr[rr] * NX + i));
+                    }
+                }
+            } else if (rok[rr]) {
+                constexpr size_t plane = (size_t)RPC * NX;
+                float *dst = part + (size_t)unit * NACC * plane + (size_t)(jr[rr] - w.y * RPC) * NX;
 #pragma unroll
                 for (int o = 0; o < NOUT; ++o) {
                     const int k1 = n2 * KPL + o / L2, k2 = o % L2;
                     const int i = 2 * (k1 + 8 * k2) + g;
-                    rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc[o], out, 0, fr.out_off + (size_t)jr[rr] * NX + i));
+#pragma unroll
+                    for (int a = 0; a < NACC; ++a) dst[a * plane + i] = acc[o][a];
                 }
             }
         }
-        block_max_to(rmax, out.fmax + w.x, wmax, NT);
+        if (split == 1) block_max_to(rmax, out.fmax + w.x, wmax, NT);
     }
     sm.release(tbase, tmem_cols<NAP, RPL, NX>());
+}
+
+// The items whose bins prop_batch_kernel split: each item's chunks added in
+// order, then the per-pixel epilogue. One warp per accumulator over 32 groups of
+// four pixels; grid.x covers an item's rows, grid.y the items.
+template <int NAP>
+__global__ void __launch_bounds__(32 * Acc<NAP>::N)
+epi_reduce_items_kernel(const float4 *__restrict__ part, const BatchFrame *__restrict__ frames,
+                        const int2 *__restrict__ items, int n_items, const int *__restrict__ n_items_dev, int sms,
+                        int cap, int nx, int rpc, EpiOut out)
+{
+    constexpr int NACC = Acc<NAP>::N;
+    if (n_items_dev) n_items = min(n_items, *n_items_dev);
+    const int split = item_split(n_items, sms, cap);
+    if (split == 1) return;
+    __shared__ float4 sA[NACC][32];
+    __shared__ float wmax[NACC];
+    const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tile4 = rpc * nx / 4;
+    const int x4 = blockIdx.x * 32 + lane, x = 4 * x4, row = x / nx, col = x - row * nx;
+    for (int it = blockIdx.y; it < n_items; it += gridDim.y) {
+        const int2 w = items[it];
+        const BatchFrame fr = frames[w.x];
+        const int j = w.y * rpc + row;
+        const bool live = x4 < tile4 && j < fr.nz;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (live) {
+            // a chunk's loads are issued 8 at a time ahead of the sums
+            const float4 *src = part + ((size_t)it * split * NACC + c) * tile4 + x4;
+            for (int s0 = 0; s0 < split; s0 += 8) {
+                float4 v[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (s0 + k < split) v[k] = src[(size_t)(s0 + k) * NACC * tile4];
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (s0 + k < split) {
+                        a.x += v[k].x; a.y += v[k].y; a.z += v[k].z; a.w += v[k].w;
+                    }
+            }
+        }
+        sA[c][lane] = a;
+        __syncthreads();
+        float rmax = 0.0f;
+        if (c == 0 && live) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float acc[NACC];
+#pragma unroll
+                for (int k = 0; k < NACC; ++k) acc[k] = reinterpret_cast<const float *>(&sA[k][lane])[i];
+                rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc, out, 0, fr.out_off + (size_t)j * nx + col + i));
+            }
+        }
+        block_max_to(rmax, out.fmax + w.x, wmax, 32 * NACC);
+        __syncthreads();
+    }
 }
 
 // Per-frame rho_n and image for a batch packed by per-frame pixel offsets.
@@ -1105,24 +1204,25 @@ cudaError_t prepare_nx()
 }
 
 template <int NAP, int NX, int RPL>
-cudaError_t launch_batch_t(int grid, const BatchFrame *frames, const int2 *items, int n_items, const int *n_items_dev,
-                           int *counter, const EpiOut &out, cudaStream_t st)
+cudaError_t launch_batch_t(const ItemWork &k, const EpiOut &out, cudaStream_t st)
 {
     static_assert(prop_smem_bytes<NAP, NX, RPL>() + 1024 <= 232448, "shared memory of the fused kernel");
-    prop_batch_kernel<NAP, NX, RPL><<<grid, 32 * prop_warps(RPL, NX), prop_smem_bytes<NAP, NX, RPL>(), st>>>(
-        frames, items, n_items, n_items_dev, counter, out);
+    prop_batch_kernel<NAP, NX, RPL><<<k.grid, 32 * prop_warps(RPL, NX), prop_smem_bytes<NAP, NX, RPL>(), st>>>(
+        k.frames, k.items, k.n_items, k.n_items_dev, k.counter, k.sms, k.cap, k.part, out);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || prop_batch_kernels(k) == 1) return e;
+    constexpr int RPC = Shape<NX, RPL>::RPC;
+    const int most = k.cap / 2 < k.n_items ? k.cap / 2 : k.n_items;   // items that can be split
+    epi_reduce_items_kernel<NAP><<<dim3((RPC * NX / 4 + 31) / 32, most), 32 * Acc<NAP>::N, 0, st>>>(
+        reinterpret_cast<const float4 *>(k.part), k.frames, k.items, k.n_items, k.n_items_dev, k.sms, k.cap, NX, RPC, out);
     return cudaGetLastError();
 }
 
 template <int NX>
-cudaError_t launch_batch_nx(int napq, int grid, const BatchFrame *frames, const int2 *items, int n_items,
-                            const int *n_items_dev, int *counter, const EpiOut &out, cudaStream_t st, int rpl)
+cudaError_t launch_batch_nx(int napq, const ItemWork &k, const EpiOut &out, cudaStream_t st, int rpl)
 {
-    if (rpl == 2)
-        return napq == 2 ? launch_batch_t<2, NX, 2>(grid, frames, items, n_items, n_items_dev, counter, out, st)
-                         : launch_batch_t<3, NX, 2>(grid, frames, items, n_items, n_items_dev, counter, out, st);
-    return napq == 2 ? launch_batch_t<2, NX, 1>(grid, frames, items, n_items, n_items_dev, counter, out, st)
-                     : launch_batch_t<3, NX, 1>(grid, frames, items, n_items, n_items_dev, counter, out, st);
+    if (rpl == 2) return napq == 2 ? launch_batch_t<2, NX, 2>(k, out, st) : launch_batch_t<3, NX, 2>(k, out, st);
+    return napq == 2 ? launch_batch_t<2, NX, 1>(k, out, st) : launch_batch_t<3, NX, 1>(k, out, st);
 }
 
 template <int NX>
@@ -1263,16 +1363,23 @@ cudaError_t launch_epilogue(const pam_plan_s &p, int n_frames, int napq, int n_s
     return cudaGetLastError();
 }
 
-cudaError_t launch_prop_batch(int nx, int napq, int grid, const BatchFrame *frames, const int2 *items, int n_items,
-                              int *counter, const EpiOut &out, cudaStream_t st, const int *n_items_dev, int rpl)
+int item_units(int n_items, int sms, int cap) { return n_items * item_split(n_items, sms, cap); }
+
+int prop_batch_kernels(const ItemWork &k)
+{
+    // with the count on the device the split is known there only
+    return k.cap >= 2 && (k.n_items_dev || item_split(k.n_items, k.sms, k.cap) > 1) ? 2 : 1;
+}
+
+cudaError_t launch_prop_batch(int nx, int napq, const ItemWork &k, const EpiOut &out, cudaStream_t st, int rpl)
 {
     if (napq != 2 && napq != 3) return cudaErrorInvalidValue;
     if (rpl != 1 && rpl != 2) return cudaErrorInvalidValue;
     switch (nx) {
-    case 16: return launch_batch_nx<16>(napq, grid, frames, items, n_items, n_items_dev, counter, out, st, rpl);
-    case 32: return launch_batch_nx<32>(napq, grid, frames, items, n_items, n_items_dev, counter, out, st, rpl);
-    case 64: return launch_batch_nx<64>(napq, grid, frames, items, n_items, n_items_dev, counter, out, st, rpl);
-    case 128: return launch_batch_nx<128>(napq, grid, frames, items, n_items, n_items_dev, counter, out, st, rpl);
+    case 16: return launch_batch_nx<16>(napq, k, out, st, rpl);
+    case 32: return launch_batch_nx<32>(napq, k, out, st, rpl);
+    case 64: return launch_batch_nx<64>(napq, k, out, st, rpl);
+    case 128: return launch_batch_nx<128>(napq, k, out, st, rpl);
     default: return cudaErrorInvalidValue;
     }
 }
