@@ -74,7 +74,6 @@ void free_plan_memory(pam_plan_s *p)
     fr(p->t.phase); fr(p->t.live); fr(p->t.bin_evan);
     fr(p->w.S); fr(p->w.Q); fr(p->w.part); fr(p->w.rho_tmp); fr(p->w.e_tmp);
     fr(p->w.fmax); fr(p->w.status); fr(p->w.rf_stage); fr(p->w.img_stage); fr(p->w.rho_stage);
-    fr(p->w.pad_img); fr(p->w.pad_rho); fr(p->w.pad_as); fr(p->w.pad_pairs);
     fr(p->t.c_hi); fr(p->t.c_lo); fr(p->t.ktab); fr(p->t.kwgt); fr(p->w.Bhi); fr(p->w.Blo); fr(p->w.smax);
     p->t = pam::Tables{};
     p->w = pam::Workspace{};
@@ -310,14 +309,6 @@ pam_status alloc_plan(pam_plan_s *p)
         PAM_TRY(cudaMemcpy(p->t.ktab, p->ktab_h.data(), p->K * sizeof(short), cudaMemcpyHostToDevice));
         PAM_TRY(cudaMemcpy(p->t.kwgt, p->kwgt_h.data(), p->K * sizeof(float), cudaMemcpyHostToDevice));
     }
-    if (p->nx_out != p->nx) {   // PAM_LATERAL_PAD2X: full-width maps, cropped after the epilogue
-        PAM_TRY(dalloc(&p->w.pad_img, F * npix));
-        if (p->n_apod >= 2) {
-            PAM_TRY(dalloc(&p->w.pad_rho, F * npix));
-            PAM_TRY(dalloc(&p->w.pad_as, F * npix));
-            PAM_TRY(dalloc(&p->w.pad_pairs, F * (p->n_apod == 3 ? 3 : 1) * npix));
-        }
-    }
     PAM_TRY(cudaMemset(p->w.status, 0, sizeof(int)));
     PAM_TRY(cudaMemcpy(p->t.bins, p->bins.data(), nb * sizeof(int), cudaMemcpyHostToDevice));
     {
@@ -364,7 +355,8 @@ pam::EpiOut epi_out(const pam_plan_s *p, float *main, float *rho_n, float *rho_p
 {
     pam::EpiOut o;
     o.eps = p->d.eps;
-    o.npix = p->nz * p->nx;
+    o.nx = p->nx_out;   // with PAM_LATERAL_PAD2X the epilogue crops
+    o.npix = p->nz * p->nx_out;
     o.out_main = main;
     o.rho_n = rho_n;
     o.rho_pairs = rho_pairs;
@@ -382,7 +374,6 @@ pam_status run_xcorr(pam_plan_t p, const float *rf, int n_frames, float *image, 
     const size_t npix = (size_t)p->nz * p->nx_out;   // caller's maps
     const size_t fr_in = (size_t)p->ne * p->nt;
     const int npairs = p->n_apod == 3 ? 3 : 1;
-    const bool crop = p->nx_out != p->nx;             // PAM_LATERAL_PAD2X
     if (pam::fault_injected("launch"))
         return fail(PAM_ERR_CUDA, "injected launch failure (PAM_FAULT=launch): nothing was queued");
     for (int f0 = 0; f0 < n_frames; f0 += p->max_frames) {
@@ -407,9 +398,7 @@ pam_status run_xcorr(pam_plan_t p, const float *rf, int n_frames, float *image, 
         e = pam::launch_lateral(*p, Fc, p->n_apod, p->t.apod, st);
         if (e != cudaSuccess) return cuda_fail(e, "lateral DFT launch");
         int ns = pam::choose_split(*p, Fc);
-        // with padding the epilogue writes full-width maps (rho_n and E always) for the crop
-        pam::EpiOut out = crop ? epi_out(p, p->w.pad_img, p->w.pad_rho, c_pairs ? p->w.pad_pairs : nullptr, p->w.pad_as)
-                               : epi_out(p, c_img, c_rho, c_pairs, c_as);
+        pam::EpiOut out = epi_out(p, c_img, c_rho, c_pairs, c_as);
         if ((e = prof_begin(p, st)) != cudaSuccess) return cuda_fail(e, "profile event");
         e = pam::launch_prop(*p, Fc, p->n_apod, ns, nullptr, out, st);
         if (e != cudaSuccess) return cuda_fail(e, "propagate/correlate launch");
@@ -417,12 +406,6 @@ pam_status run_xcorr(pam_plan_t p, const float *rf, int n_frames, float *image, 
         e = pam::launch_epilogue(*p, Fc, p->n_apod, ns, out, st);
         if (e != cudaSuccess) return cuda_fail(e, "epilogue launch");
         p->kernels += 3 + pam::epilogue_kernels(*p, p->n_apod, ns);
-        if (crop) {
-            e = pam::launch_pad_crop(p->w.pad_rho, p->w.pad_as, p->w.pad_pairs, npairs, Fc, p->nz, p->nx, p->nx_out,
-                                     c_img, c_rho, c_pairs, c_as, st);
-            if (e != cudaSuccess) return cuda_fail(e, "crop launch");
-            p->kernels += 1;
-        }
     }
     return PAM_OK;
 }
@@ -513,8 +496,7 @@ pam_status pam_as_backprop(pam_plan_t p, const float *rf, int n_frames, int apod
     if ((s = check_dev_ptr(rf, "rf", true)) != PAM_OK) return s;
     if ((s = check_dev_ptr(energy, "energy", true)) != PAM_OK) return s;
     if ((s = check_dev_ptr(fields, "fields", false)) != PAM_OK) return s;
-    const bool crop = p->nx_out != p->nx;   // PAM_LATERAL_PAD2X
-    if (fields && crop) return fail(PAM_ERR_UNSUPPORTED, "the fields output is not built with PAM_LATERAL_PAD2X");
+    if (fields && p->nx_out != p->nx) return fail(PAM_ERR_UNSUPPORTED, "the fields output is not built with PAM_LATERAL_PAD2X");
     if (pam::fault_injected("launch"))
         return fail(PAM_ERR_CUDA, "injected launch failure (PAM_FAULT=launch): nothing was queued");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -529,7 +511,7 @@ pam_status pam_as_backprop(pam_plan_t p, const float *rf, int n_frames, int apod
         if (e != cudaSuccess) return cuda_fail(e, "lateral DFT launch");
         int ns = pam::choose_split(*p, Fc);
         float *fl = fields ? fields + (size_t)f0 * p->n_bins * npix * 2 : nullptr;
-        pam::EpiOut out = epi_out(p, crop ? p->w.pad_img : energy + (size_t)f0 * npix, nullptr, nullptr, nullptr);
+        pam::EpiOut out = epi_out(p, energy + (size_t)f0 * npix, nullptr, nullptr, nullptr);
         if ((e = prof_begin(p, st)) != cudaSuccess) return cuda_fail(e, "profile event");
         e = pam::launch_prop(*p, Fc, 1, ns, fl, out, st);
         if (e != cudaSuccess) return cuda_fail(e, "propagate launch");
@@ -537,12 +519,6 @@ pam_status pam_as_backprop(pam_plan_t p, const float *rf, int n_frames, int apod
         e = pam::launch_epilogue(*p, Fc, 1, ns, out, st, false, fl != nullptr);
         if (e != cudaSuccess) return cuda_fail(e, "epilogue launch");
         p->kernels += 3 + pam::epilogue_kernels(*p, 1, ns, fl != nullptr);
-        if (crop) {   // element columns of the padded energy map
-            const size_t w_out = (size_t)p->nx_out * sizeof(float), w_in = (size_t)p->nx * sizeof(float);
-            e = cudaMemcpy2DAsync(energy + (size_t)f0 * npix, w_out, p->w.pad_img, w_in, w_out, (size_t)Fc * p->nz,
-                                  cudaMemcpyDeviceToDevice, st);
-            if (e != cudaSuccess) return cuda_fail(e, "crop copy");
-        }
     }
     return PAM_OK;
 }

@@ -338,7 +338,7 @@ pam_status enqueue(pam_batch_s *b, const float *rf, float *image, float *rho_n, 
         return pam::cuda_fail(e, "memset");
     pam::EpiOut out;
     out.eps = p.d.eps;
-    out.npix = 0;
+    out.nx = b->nx;
     out.out_main = image;
     out.rho_n = rho_n;
     out.rho_tmp = p.w.rho_tmp;

@@ -33,6 +33,7 @@ inline size_t q_per_bin(int napq, int nx) { return (size_t)2 * napq * nx; }
 // Destination of the per-pixel epilogue (maps of one call, [F][nz][nx]).
 struct EpiOut {
     float eps = 1e-3f;
+    int nx = 0;                   // image columns (columns past them are not written)
     int npix = 0;                 // nz * nx
     float *out_main = nullptr;    // AS energy (n_apod 1) or the final image (DAX / TAX)
     float *rho_n = nullptr;       // optional
@@ -87,9 +88,6 @@ struct Workspace {
     unsigned *smax = nullptr;               // [max_frames] max |Re S|, |Im S| bits
     // host-buffer entry point staging (allocated on first use)
     float *rf_stage = nullptr, *img_stage = nullptr, *rho_stage = nullptr;
-    // PAM_LATERAL_PAD2X: full-width maps before the crop, [max_frames][npix] each
-    // (pad_pairs: [max_frames][pairs][npix]; only pad_img for n_apod == 1)
-    float *pad_img = nullptr, *pad_rho = nullptr, *pad_as = nullptr, *pad_pairs = nullptr;
 };
 
 struct Tables {
@@ -192,14 +190,6 @@ cudaError_t launch_normalize_batch(int n_frames, int max_npix, const BatchFrame 
 bool prop_uses_cluster(int n_split);
 // A kernel whose bounded mbarrier wait never completes (failure-path test).
 cudaError_t launch_expire_wait(int *status, cudaStream_t st);
-
-// PAM_LATERAL_PAD2X crop: columns [0, nx_out) of the full-width maps (row
-// width nx) of n_frames frames. rho_n is renormalised to its maximum over the
-// crop and the image rebuilt as rho_n^2 E from the full-aperture energy E.
-// Outputs other than image may be NULL.
-cudaError_t launch_pad_crop(const float *rho_full, const float *e_full, const float *pairs_full, int n_pairs,
-                            int n_frames, int nz, int nx, int nx_out, float *image, float *rho_n, float *pairs,
-                            float *image_as, cudaStream_t st);
 
 // Host-side fault injection for tests: true when the environment variable
 // PAM_FAULT names `what` ("alloc": plan allocation fails part way).

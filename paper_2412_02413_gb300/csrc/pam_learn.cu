@@ -1147,6 +1147,7 @@ pam_status pam_learn_example(pam_learn_t l, const float *rf, int n_frames, void 
         LTRY(cudaGetLastError());
         pam::EpiOut out;
         out.eps = p.d.eps;
+        out.nx = l->W;
         out.rho_tmp = target;
         out.e_tmp = p.w.e_tmp;
         out.fmax = l->fmax_x;
@@ -1249,6 +1250,7 @@ pam_status pam_learn_tax(pam_learn_t l, const float *rf, int n_frames, float *im
         LTRY(pam::launch_lateral(p, n, 3, p.t.apod, st));
         pam::EpiOut out;
         out.eps = p.d.eps;
+        out.nx = l->W;
         out.rho_tmp = p.w.rho_tmp;
         out.e_tmp = p.w.e_tmp;
         out.fmax = l->fmax_g;

@@ -180,12 +180,17 @@ __device__ __forceinline__ float ncc_pair(float c, float aq, float ar, float eps
 // AS (Eq. 3): the energy itself. AS-DAX / AS-TAX: the clamped pair NCCs, rho
 // (rho_12, or Eq. 10's cube root of the three), and the coherent energy
 // E = sum_k |sum_q p_q|^2 = sum A_qq + 2 sum C_qr. Writes the
-// pre-normalisation maps and returns rho (0 for AS).
+// pre-normalisation maps of the frame whose maps start at pixel `base` and
+// returns rho (0 for AS). Columns past the image (PAM_LATERAL_PAD2X computes 2 ne
+// of them and keeps ne) are dropped here, so the maps are cropped as they are
+// written and rho's maximum is the crop's; a crop of full-width maps afterwards,
+// one CTA per frame, took 38 us for three 64 x 128 frames.
 template <int NAP>
-__device__ __forceinline__ float pixel_epilogue(const float (&a)[Acc<NAP>::N], const EpiOut &out, int f,
-                                                size_t x)
+__device__ __forceinline__ float pixel_epilogue(const float (&a)[Acc<NAP>::N], const EpiOut &out, size_t base,
+                                                int row, int col)
 {
-    const size_t o = (size_t)f * out.npix + x;
+    if (col >= out.nx) return 0.0f;
+    const size_t o = base + (size_t)row * out.nx + col;
     if constexpr (NAP == 1) {
         out.out_main[o] = a[0];
         return 0.0f;
@@ -200,7 +205,7 @@ __device__ __forceinline__ float pixel_epilogue(const float (&a)[Acc<NAP>::N], c
             const float r23 = ncc_pair(a[4], a[1], a[2], out.eps);
             const float r31 = ncc_pair(a[5], a[2], a[0], out.eps);
             if (out.rho_pairs) {
-                float *rp = out.rho_pairs + (size_t)f * 3 * out.npix + x;
+                float *rp = out.rho_pairs + 2 * base + o;   // three planes per frame
                 rp[0] = r12;
                 rp[out.npix] = r23;
                 rp[2 * (size_t)out.npix] = r31;
@@ -656,7 +661,7 @@ prop_corr_kernel(const float2 *__restrict__ Q, const uint4 *__restrict__ phase,
                 for (int aa = 0; aa < NACC; ++aa) a[aa] += rem[aa * TILE + px];
             }
             const int row = blockIdx.x * RPC + px / NX;
-            if (row < nz && !aborted) rmax = fmaxf(rmax, pixel_epilogue<NAP>(a, out, f, (size_t)row * NX + (px % NX)));
+            if (row < nz && !aborted) rmax = fmaxf(rmax, pixel_epilogue<NAP>(a, out, (size_t)f * out.npix, row, px % NX));
         }
         if constexpr (NAP > 1) {
             __shared__ float wmax[PROP_THREADS / 32];
@@ -758,7 +763,7 @@ prop_seg_kernel(const float2 *__restrict__ Q, const uint4 *__restrict__ phase, c
                     for (int o = 0; o < NOUT; ++o) {
                         const int k1 = n2 * KPL + o / L2, k2 = o % L2;
                         const int i = 2 * (k1 + 8 * k2) + g;
-                        rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc[o], out, f, (size_t)jr[rr] * NX + i));
+                        rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc[o], out, (size_t)f * out.npix, jr[rr], i));
                     }
                 }
             } else if (rok[rr]) {
@@ -791,7 +796,7 @@ constexpr int EPI_THREADS = 128;
 // sums.
 template <int NAP>
 __global__ void __launch_bounds__(EPI_THREADS)
-epi_reduce_kernel(const float4 *__restrict__ part, int n_split, int npix4, EpiOut out)
+epi_reduce_kernel(const float4 *__restrict__ part, int n_split, int npix4, int nx, EpiOut out)
 {
     constexpr int NACC = Acc<NAP>::N;
     __shared__ float wmax[EPI_THREADS / 32];
@@ -817,7 +822,7 @@ epi_reduce_kernel(const float4 *__restrict__ part, int n_split, int npix4, EpiOu
             float acc[NACC];
 #pragma unroll
             for (int k = 0; k < NACC; ++k) acc[k] = reinterpret_cast<const float *>(&a[k])[i];
-            rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc, out, f, (size_t)x4 * 4 + i));
+            rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc, out, (size_t)f * out.npix, 4 * x4 / nx, 4 * x4 % nx + i));
         }
     }
     if constexpr (NAP > 1) block_max_to(rmax, out.fmax + f, wmax, EPI_THREADS);
@@ -879,17 +884,19 @@ epi_reduce_seg_kernel(const float4 *__restrict__ part, int npix4, int nx, int rp
             float acc[NACC];
 #pragma unroll
             for (int k = 0; k < NACC; ++k) acc[k] = reinterpret_cast<const float *>(&sA[k][lane])[i];
-            rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc, out, f, (size_t)x4 * 4 + i));
+            rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc, out, (size_t)f * out.npix, 4 * x4 / nx, 4 * x4 % nx + i));
         }
     }
     if constexpr (NAP > 1) block_max_to(rmax, out.fmax + f, wmax, 32 * NACC);
 }
 
 // rho_n = rho / max (Sec. II-A: the maximum becomes exactly 1) and the image
-// I = rho_n^2 E (Eq. 5 / Eq. 11). Four pixels per thread.
+// I = rho_n^2 E (Eq. 5 / Eq. 11). Four pixels per thread. `guard`: a maximum that
+// is not positive (a frame without a finite rho) gives rho_n = 0, the reading of
+// the padded maps; without it the division's result stands.
 __global__ void __launch_bounds__(EPI_THREADS)
 epi_normalize_kernel(const float4 *__restrict__ rho_tmp, const float4 *__restrict__ e_tmp,
-                     const unsigned *__restrict__ fmax, int npix4, float4 *__restrict__ image,
+                     const unsigned *__restrict__ fmax, int npix4, bool guard, float4 *__restrict__ image,
                      float4 *__restrict__ rho_n)
 {
     const int f = blockIdx.y;
@@ -898,7 +905,8 @@ epi_normalize_kernel(const float4 *__restrict__ rho_tmp, const float4 *__restric
     const size_t o = (size_t)f * npix4 + x;
     const float m = __uint_as_float(fmax[f]);
     const float4 r = rho_tmp[o], e = e_tmp[o];
-    const float4 rn = make_float4(r.x / m, r.y / m, r.z / m, r.w / m);
+    float4 rn = make_float4(r.x / m, r.y / m, r.z / m, r.w / m);
+    if (guard && !(m > 0.0f)) rn = make_float4(0.f, 0.f, 0.f, 0.f);
     image[o] = make_float4(rn.x * rn.x * e.x, rn.y * rn.y * e.y, rn.z * rn.z * e.z, rn.w * rn.w * e.w);
     if (rho_n) rho_n[o] = rn;
 }
@@ -994,7 +1002,7 @@ prop_batch_kernel(const BatchFrame *__restrict__ frames, const int2 *__restrict_
                     for (int o = 0; o < NOUT; ++o) {
                         const int k1 = n2 * KPL + o / L2, k2 = o % L2;
                         const int i = 2 * (k1 + 8 * k2) + g;
-                        rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc[o], out, 0, fr.out_off + (size_t)jr[rr] * NX + i));
+                        rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc[o], out, fr.out_off, jr[rr], i));
                     }
                 }
             } else if (rok[rr]) {
@@ -1062,7 +1070,7 @@ epi_reduce_items_kernel(const float4 *__restrict__ part, const BatchFrame *__res
                 float acc[NACC];
 #pragma unroll
                 for (int k = 0; k < NACC; ++k) acc[k] = reinterpret_cast<const float *>(&sA[k][lane])[i];
-                rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc, out, 0, fr.out_off + (size_t)j * nx + col + i));
+                rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc, out, fr.out_off, j, col + i));
             }
         }
         block_max_to(rmax, out.fmax + w.x, wmax, 32 * NACC);
@@ -1349,17 +1357,18 @@ cudaError_t launch_epilogue(const pam_plan_s &p, int n_frames, int napq, int n_s
     } else if (from_partials || !prop_uses_cluster(n_split)) {
         const float4 *part = reinterpret_cast<const float4 *>(p.w.part);
         if (napq == 1)
-            epi_reduce_kernel<1><<<grid, EPI_THREADS, 0, st>>>(part, n_split, npix4, out);
+            epi_reduce_kernel<1><<<grid, EPI_THREADS, 0, st>>>(part, n_split, npix4, p.nx, out);
         else if (napq == 2)
-            epi_reduce_kernel<2><<<grid, EPI_THREADS, 0, st>>>(part, n_split, npix4, out);
+            epi_reduce_kernel<2><<<grid, EPI_THREADS, 0, st>>>(part, n_split, npix4, p.nx, out);
         else
-            epi_reduce_kernel<3><<<grid, EPI_THREADS, 0, st>>>(part, n_split, npix4, out);
+            epi_reduce_kernel<3><<<grid, EPI_THREADS, 0, st>>>(part, n_split, npix4, p.nx, out);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     if (napq == 1) return cudaSuccess;
-    epi_normalize_kernel<<<grid, EPI_THREADS, 0, st>>>(v4(out.rho_tmp), v4(out.e_tmp), out.fmax, npix4,
-                                                       v4(out.out_main), v4(out.rho_n));
+    const int out4 = out.npix / 4;      // the image's pixels (fewer than npix4 with padding)
+    epi_normalize_kernel<<<dim3((out4 + EPI_THREADS - 1) / EPI_THREADS, n_frames), EPI_THREADS, 0, st>>>(
+        v4(out.rho_tmp), v4(out.e_tmp), out.fmax, out4, out.nx != p.nx, v4(out.out_main), v4(out.rho_n));
     return cudaGetLastError();
 }
 

@@ -217,6 +217,7 @@ extern "C" pam_status pam_as_tax_static(const pam_plan_desc *d, const float *rf,
         if ((e = pam::launch_lateral(p, 1, 3, p.t.apod, st)) != cudaSuccess) return cuda_fail(e, "lateral DFT");
         pam::EpiOut out;
         out.eps = d->eps;
+        out.nx = nx;
         out.npix = (int)npix;
         out.out_main = image_tax + f * npix;
         out.rho_n = rho_n ? rho_n + f * npix : nullptr;
