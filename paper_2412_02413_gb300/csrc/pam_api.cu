@@ -368,6 +368,18 @@ pam::EpiOut epi_out(const pam_plan_s *p, float *main, float *rho_n, float *rho_p
     return o;
 }
 
+// Whether a call's kernels may overlap each other's launches: not while the
+// stream is being captured, where the plain dependencies are kept.
+bool overlap_launches(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+        cudaGetLastError();   // the launches report what is wrong
+        return false;
+    }
+    return cs == cudaStreamCaptureStatusNone;
+}
+
 pam_status run_xcorr(pam_plan_t p, const float *rf, int n_frames, float *image, float *rho_n,
                      float *rho_pairs, float *image_as, cudaStream_t st)
 {
@@ -376,6 +388,7 @@ pam_status run_xcorr(pam_plan_t p, const float *rf, int n_frames, float *image, 
     const int npairs = p->n_apod == 3 ? 3 : 1;
     if (pam::fault_injected("launch"))
         return fail(PAM_ERR_CUDA, "injected launch failure (PAM_FAULT=launch): nothing was queued");
+    p->pdl = overlap_launches(st);
     for (int f0 = 0; f0 < n_frames; f0 += p->max_frames) {
         int Fc = std::min(p->max_frames, n_frames - f0);
         float *c_img = image + (size_t)f0 * npix, *c_rho = rho_n ? rho_n + (size_t)f0 * npix : nullptr;
@@ -500,6 +513,7 @@ pam_status pam_as_backprop(pam_plan_t p, const float *rf, int n_frames, int apod
     if (pam::fault_injected("launch"))
         return fail(PAM_ERR_CUDA, "injected launch failure (PAM_FAULT=launch): nothing was queued");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    p->pdl = overlap_launches(st);
     const float *apod = apod_index < 0 ? p->t.ones : p->t.apod + (size_t)apod_index * p->nev;
     const size_t npix = (size_t)p->nz * p->nx_out;
     const size_t fr_in = (size_t)p->ne * p->nt;

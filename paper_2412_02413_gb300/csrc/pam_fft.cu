@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "pam_internal.h"
+#include "pam_ptx.h"
 
 namespace pam {
 namespace {
@@ -213,12 +214,14 @@ time_fft_kernel(const float *__restrict__ rf, int ne, int nt, int log2nt, const 
     float2 *x = sbuf, *y = sbuf + M, *tws = sbuf + 2 * M;
     const int f = blockIdx.y, e = blockIdx.x;
     const float4 *src = reinterpret_cast<const float4 *>(rf + ((size_t)f * ne + e) * nt);
-    if (e == 0 && threadIdx.x == 0) fmax[f] = 0u;
     float4 *x4 = reinterpret_cast<float4 *>(x);
+    for (int m = threadIdx.x; m < M; m += TFFT_THREADS) tws[m] = tw[2 * m];    // exp(-2 pi i m / M), a plan table
+    ptx::pdl_wait();
+    if (e == 0 && threadIdx.x == 0) fmax[f] = 0u;
     for (int i = threadIdx.x; i < nt / 4; i += TFFT_THREADS) x4[i] = src[i];  // (x0,x1),(x2,x3) pairs
-    for (int m = threadIdx.x; m < M; m += TFFT_THREADS) tws[m] = tw[2 * m];    // exp(-2 pi i m / M)
     __syncthreads();
     float2 *Z = stockham<MAXR>(x, y, M, log2nt - 1, 1, tws, threadIdx.x, TFFT_THREADS);
+    ptx::pdl_trigger();
     for (int b = threadIdx.x; b < n_bins; b += TFFT_THREADS) {
         const int k = bins[b];                                 // 0 < k < M
         const float2 zk = Z[k], zm = Z[M - k];
@@ -255,15 +258,17 @@ lateral_kernel(const float2 *__restrict__ S, int ne, int nx, int log2nx, int n_b
     float2 *x = lbuf, *y = lbuf + napq * nx, *tws = lbuf + 2 * napq * nx;
     const int f = blockIdx.y, b = blockIdx.x;
     const float2 *s = S + ((size_t)f * n_bins + b) * ne;
+    for (int i = threadIdx.x; i < nx; i += LAT_THREADS) tws[i] = twx[i];   // a plan table
+    ptx::pdl_wait();
     for (int i = threadIdx.x; i < napq * nx; i += LAT_THREADS) {
         const int q = i / nx, e = i - q * nx;
         const float2 v = s[e];
         const float a = apod[q * ne + e];
         x[i] = make_float2(a * v.x, a * v.y);
     }
-    for (int i = threadIdx.x; i < nx; i += LAT_THREADS) tws[i] = twx[i];
     __syncthreads();
     const float2 *X = stockham<4>(x, y, nx, log2nx, napq, tws, threadIdx.x, LAT_THREADS);
+    ptx::pdl_trigger();
     const float inv_nx = 1.0f / (float)nx;
     float2 *dst = Q + ((size_t)f * n_bins + b) * (2 * napq * nx);
     const int H = nx / 2, L2 = nx / 16;
@@ -312,17 +317,15 @@ cudaError_t launch_time_fft(const pam_plan_s &p, const float *rf, int n_frames, 
 {
     dim3 grid(p.ne, n_frames);
     auto kern = p.fft_radix == 8 ? time_fft_kernel<8> : time_fft_kernel<4>;
-    kern<<<grid, TFFT_THREADS, time_fft_smem(p.nt), st>>>(rf, p.ne, p.nt, ilog2i(p.nt), p.t.tw_t, p.t.bins,
-                                                          p.n_bins, p.w.S, p.nev, p.chan_step, p.w.fmax);
-    return cudaGetLastError();
+    return launch_pdl(p.pdl, kern, grid, TFFT_THREADS, time_fft_smem(p.nt), st, rf, p.ne, p.nt, ilog2i(p.nt), p.t.tw_t,
+                      p.t.bins, p.n_bins, p.w.S, p.nev, p.chan_step, p.w.fmax);
 }
 
 cudaError_t launch_lateral(const pam_plan_s &p, int n_frames, int napq, const float *apod, cudaStream_t st)
 {
     dim3 grid(p.n_bins, n_frames);
-    lateral_kernel<<<grid, LAT_THREADS, lateral_smem(p.nx, napq), st>>>(p.w.S, p.nev, p.nx, ilog2i(p.nx), p.n_bins,
-                                                                        napq, apod, p.t.tw_x, p.t.live, 0, p.w.Q);
-    return cudaGetLastError();
+    return launch_pdl(p.pdl, lateral_kernel, grid, LAT_THREADS, lateral_smem(p.nx, napq), st, p.w.S, p.nev, p.nx,
+                      ilog2i(p.nx), p.n_bins, napq, apod, p.t.tw_x, p.t.live, 0, p.w.Q);
 }
 
 cudaError_t launch_lateral_frames(const pam_plan_s &p, int n_frames, int napq, const float *apod,

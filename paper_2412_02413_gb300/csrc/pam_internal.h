@@ -136,6 +136,7 @@ struct pam_plan_s {
     int lane_rows = 2;                 // pam_plan_set_lane_rows: depth rows per lane of the fused kernel (1 or 2)
     int gemm_m = 128;                  // pam_plan_set_gemm_tile: M of the tensor-core form's MMA (128 or 256)
     int gemm_frames = 32;              // pam_plan_set_gemm_frames: frames per CTA of the tensor-core form (32 or 16)
+    bool pdl = false;                  // this call's kernels overlap each other's launches (set per call)
     bool seg_ok = false;               // Workspace::part holds prop_seg_part_floats (even division of small batches)
     // tensor-core form (PAM_FORM_GEMM_*): 0 = plain FP32 path
     int form = 0;
@@ -146,6 +147,27 @@ struct pam_plan_s {
 };
 
 namespace pam {
+
+// Launch with programmatic stream serialisation where `pdl` is set: the kernel
+// (which calls ptx::pdl_wait) may start its set-up while the previous kernel of
+// the stream drains.
+template <class... P, class... A>
+cudaError_t launch_pdl(bool pdl, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    if (pdl) {
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+    }
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
 
 // Launchers (all asynchronous on `st`). Each returns cudaGetLastError().
 cudaError_t launch_tables(const pam_plan_s &p, cudaStream_t st);

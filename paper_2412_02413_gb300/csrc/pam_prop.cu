@@ -726,6 +726,7 @@ prop_seg_kernel(const float2 *__restrict__ Q, const uint4 *__restrict__ phase, c
     const int r = lane / LPR, g = (lane % LPR) / L2, n2 = lane % L2;
     const unsigned tbase = sm.init(tmem_cols<NAP, RPL, NX>());
     const unsigned tcol = acc_tcol(tbase, warp, NACC, RPL);
+    pdl_wait();
     const int G = gridDim.x, c = blockIdx.x;
     long long w = (long long)c * W / G;
     const long long w1 = (long long)(c + 1) * W / G;
@@ -751,6 +752,7 @@ prop_seg_kernel(const float2 *__restrict__ Q, const uint4 *__restrict__ phase, c
         seq += (unsigned)nb;
         if (!ok && lane == 0) atomicOr(out.status, 1);
         if (__syncthreads_or(!ok)) break;
+        if (w + nb >= w1) pdl_trigger();   // the last segment's sums are still to be written
         float rmax = 0.0f;
 #pragma unroll
         for (int rr = 0; rr < RPL; ++rr) {
@@ -832,62 +834,65 @@ epi_reduce_kernel(const float4 *__restrict__ part, int n_split, int npix4, int n
 // more CTAs share, its slots added in CTA order (deterministic), then the
 // per-pixel epilogue. A tile inside one CTA's share was finished by that CTA;
 // its blocks return at once (a block's 128 pixels never straddle tiles).
-// Layout as epi_reduce_kernel: one warp per accumulator over 32 groups of four
-// pixels.
+// One warp per accumulator adds 32 groups of four pixels; then four warps (of AS:
+// one) finish a pixel per thread. Bound by the latency of the slots' loads (L2)
+// and of the square roots, divisions and the cube root behind them.
 template <int NAP>
-__global__ void __launch_bounds__(32 * Acc<NAP>::N)
+__global__ void __launch_bounds__(Acc<NAP>::N < 4 ? 128 : 32 * Acc<NAP>::N)
 epi_reduce_seg_kernel(const float4 *__restrict__ part, int npix4, int nx, int rpc, int n_bins, int tiles, long long W,
                       int G, EpiOut out)
 {
-    constexpr int NACC = Acc<NAP>::N;
+    constexpr int NACC = Acc<NAP>::N, NT = NACC < 4 ? 128 : 32 * NACC;
     __shared__ float4 sA[NACC][32];
-    __shared__ float wmax[NACC];
+    __shared__ float wmax[NT / 32];
     const int f = blockIdx.y;
     const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tile4 = rpc * nx / 4;                    // float4 groups per tile
     const int tile = (blockIdx.x * 32) / tile4;
     const long long tt = (long long)f * tiles + tile;
     const int cf = seg_cta_of(tt * n_bins, W, G), cl = seg_cta_of((tt + 1) * n_bins - 1, W, G);
+    // CTAs cf < cc <= cl start inside this tile (their first segment, slot
+    // 2 cc); cf's segment is its last unless its share starts at this tile.
+    const int cf_slot = 2 * cf + ((tt > 0 && seg_cta_of(tt * n_bins - 1, W, G) == cf) ? 1 : 0);
+    pdl_wait();
     if (cf == cl) return;                              // block-uniform
     const int x4 = blockIdx.x * 32 + lane;
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (x4 < npix4) {
-        // CTAs cf < cc <= cl start inside this tile (their first segment, slot
-        // 2 cc); cf's segment is its last unless its share starts at this tile.
-        // The slots' loads are all issued before the sums (in CTA order), in
-        // batches of 16, so that their latencies overlap.
-        constexpr int MAXS = 16;
-        const int cf_slot = 2 * cf + ((tt > 0 && seg_cta_of(tt * n_bins - 1, W, G) == cf) ? 1 : 0);
-        const size_t off = (size_t)c * tile4 + (x4 - tile * tile4);
-        const int ns = cl - cf + 1;
-        for (int base = 0; base < ns; base += MAXS) {
-            float4 v[MAXS];
+    if (c < NACC) {
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (x4 < npix4) {
+            // The slots' loads are all issued before the sums (in CTA order), in
+            // batches of 16, so that their latencies overlap.
+            constexpr int MAXS = 16;
+            const size_t off = (size_t)c * tile4 + (x4 - tile * tile4);
+            const int ns = cl - cf + 1;
+            for (int base = 0; base < ns; base += MAXS) {
+                float4 v[MAXS];
 #pragma unroll
-            for (int k = 0; k < MAXS; ++k) {
-                const int cc = cf + base + k;
-                const size_t slot = cc == cf ? (size_t)cf_slot : 2 * (size_t)cc;
-                if (base + k < ns) v[k] = part[slot * NACC * tile4 + off];
-            }
-#pragma unroll
-            for (int k = 0; k < MAXS; ++k)
-                if (base + k < ns) {
-                    a.x += v[k].x; a.y += v[k].y; a.z += v[k].z; a.w += v[k].w;
+                for (int k = 0; k < MAXS; ++k) {
+                    const int cc = cf + base + k;
+                    const size_t slot = cc == cf ? (size_t)cf_slot : 2 * (size_t)cc;
+                    if (base + k < ns) v[k] = part[slot * NACC * tile4 + off];
                 }
+#pragma unroll
+                for (int k = 0; k < MAXS; ++k)
+                    if (base + k < ns) {
+                        a.x += v[k].x; a.y += v[k].y; a.z += v[k].z; a.w += v[k].w;
+                    }
+            }
         }
+        sA[c][lane] = a;
     }
-    sA[c][lane] = a;
+    pdl_trigger();
     __syncthreads();
     float rmax = 0.0f;
-    if (c == 0 && x4 < npix4) {
+    const int x = 128 * blockIdx.x + threadIdx.x;      // pixel of the full-width row grid
+    if (threadIdx.x < 128 && x < 4 * npix4) {
+        float acc[NACC];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float acc[NACC];
-#pragma unroll
-            for (int k = 0; k < NACC; ++k) acc[k] = reinterpret_cast<const float *>(&sA[k][lane])[i];
-            rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc, out, (size_t)f * out.npix, 4 * x4 / nx, 4 * x4 % nx + i));
-        }
+        for (int k = 0; k < NACC; ++k) acc[k] = reinterpret_cast<const float *>(&sA[k][0])[threadIdx.x];
+        rmax = pixel_epilogue<NAP>(acc, out, (size_t)f * out.npix, x / nx, x % nx);
     }
-    if constexpr (NAP > 1) block_max_to(rmax, out.fmax + f, wmax, 32 * NACC);
+    if constexpr (NAP > 1) block_max_to(rmax, out.fmax + f, wmax, NT);
 }
 
 // rho_n = rho / max (Sec. II-A: the maximum becomes exactly 1) and the image
@@ -901,6 +906,7 @@ epi_normalize_kernel(const float4 *__restrict__ rho_tmp, const float4 *__restric
 {
     const int f = blockIdx.y;
     const int x = blockIdx.x * EPI_THREADS + threadIdx.x;
+    pdl_wait();
     if (x >= npix4) return;
     const size_t o = (size_t)f * npix4 + x;
     const float m = __uint_as_float(fmax[f]);
@@ -1129,9 +1135,9 @@ cudaError_t launch_seg_rt(const pam_plan_s &p, int n_frames, const EpiOut &out, 
     const int tiles = (p.nz + S::RPC - 1) / S::RPC;
     const long long W = (long long)n_frames * tiles * p.n_bins;
     const int G = prop_seg_ctas(p, n_frames);
-    prop_seg_kernel<NAP, NX, RPL><<<G, 32 * prop_warps(RPL, NX), prop_smem_bytes<NAP, NX, RPL>(), st>>>(
-        p.w.Q, p.t.phase, p.t.bin_evan, p.n_bins, p.nz, tiles, (float)p.d.z0_m, (float)p.d.dz_m, W, p.w.part, out);
-    return cudaGetLastError();
+    return launch_pdl(p.pdl, prop_seg_kernel<NAP, NX, RPL>, G, 32 * prop_warps(RPL, NX), prop_smem_bytes<NAP, NX, RPL>(),
+                      st, p.w.Q, p.t.phase, p.t.bin_evan, p.n_bins, p.nz, tiles, (float)p.d.z0_m, (float)p.d.dz_m, W,
+                      p.w.part, out);
 }
 
 template <int NAP, int NX>
@@ -1346,13 +1352,9 @@ cudaError_t launch_epilogue(const pam_plan_s &p, int n_frames, int napq, int n_s
         const int G = prop_seg_ctas(p, n_frames);
         const float4 *part = reinterpret_cast<const float4 *>(p.w.part);
         dim3 rgrid((npix4 + 31) / 32, n_frames);
-        if (napq == 1)
-            epi_reduce_seg_kernel<1><<<rgrid, 32 * Acc<1>::N, 0, st>>>(part, npix4, p.nx, rows, p.n_bins, tiles, W, G, out);
-        else if (napq == 2)
-            epi_reduce_seg_kernel<2><<<rgrid, 32 * Acc<2>::N, 0, st>>>(part, npix4, p.nx, rows, p.n_bins, tiles, W, G, out);
-        else
-            epi_reduce_seg_kernel<3><<<rgrid, 32 * Acc<3>::N, 0, st>>>(part, npix4, p.nx, rows, p.n_bins, tiles, W, G, out);
-        cudaError_t e = cudaGetLastError();
+        auto reduce = napq == 1 ? epi_reduce_seg_kernel<1> : napq == 2 ? epi_reduce_seg_kernel<2> : epi_reduce_seg_kernel<3>;
+        cudaError_t e = launch_pdl(p.pdl, reduce, rgrid, napq == 3 ? 32 * Acc<3>::N : 128, 0, st, part, npix4, p.nx, rows,
+                                   p.n_bins, tiles, W, G, out);
         if (e != cudaSuccess) return e;
     } else if (from_partials || !prop_uses_cluster(n_split)) {
         const float4 *part = reinterpret_cast<const float4 *>(p.w.part);
@@ -1367,9 +1369,8 @@ cudaError_t launch_epilogue(const pam_plan_s &p, int n_frames, int napq, int n_s
     }
     if (napq == 1) return cudaSuccess;
     const int out4 = out.npix / 4;      // the image's pixels (fewer than npix4 with padding)
-    epi_normalize_kernel<<<dim3((out4 + EPI_THREADS - 1) / EPI_THREADS, n_frames), EPI_THREADS, 0, st>>>(
-        v4(out.rho_tmp), v4(out.e_tmp), out.fmax, out4, out.nx != p.nx, v4(out.out_main), v4(out.rho_n));
-    return cudaGetLastError();
+    return launch_pdl(p.pdl, epi_normalize_kernel, dim3((out4 + EPI_THREADS - 1) / EPI_THREADS, n_frames), EPI_THREADS, 0,
+                      st, v4(out.rho_tmp), v4(out.e_tmp), out.fmax, out4, out.nx != p.nx, v4(out.out_main), v4(out.rho_n));
 }
 
 int item_units(int n_items, int sms, int cap) { return n_items * item_split(n_items, sms, cap); }

@@ -78,6 +78,16 @@ __device__ __forceinline__ bool mbar_wait_sleep(uint64_t *bar, unsigned parity)
     return true;
 }
 
+// ---- programmatic dependent launch ----
+// Waits until the kernels this one depends on have completed and their writes
+// are visible (returns at once in a kernel launched without the attribute).
+// Every global read of their results and every global write comes after it.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+// The next kernel of the stream may be scheduled from here on (its pdl_wait
+// still waits for this one's end). Called near a kernel's end, so that the
+// dependents do not hold SMs that other streams could use.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
 // ---- thread-block clusters ----
 __device__ __forceinline__ unsigned cluster_ctarank()
 {
