@@ -145,17 +145,26 @@ def _check(status: int):
         raise PamError(status, msg)
 
 
+_torch = None   # the torch module, once it has been seen to have a GPU
+
+
 def _require_cuda():
-    import torch
-    if not torch.cuda.is_available():
-        raise RuntimeError("libpam needs a CUDA GPU; no CPU fallback exists")
-    return torch
+    global _torch
+    if _torch is None:
+        import torch
+        if not torch.cuda.is_available():
+            raise RuntimeError("libpam needs a CUDA GPU; no CPU fallback exists")
+        _torch = torch
+    return _torch
 
 
 def _stream_ptr(stream=None) -> int:
+    # the raw handle of the current stream: building torch's stream object to ask
+    # it took 3.9 us of a one-frame call's 16 us of Python
+    if stream is not None:
+        return int(stream.cuda_stream)
     torch = _require_cuda()
-    s = torch.cuda.current_stream() if stream is None else stream
-    return int(s.cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _dptr(t) -> Optional[int]:
