@@ -131,13 +131,23 @@ template <int NX, int RPL = 1> struct Shape {
     static constexpr int RPW = 32 / LPR * RPL;     // rows per warp
     static constexpr int RPC = prop_warps(RPL, NX) * RPW;   // rows per CTA
     static constexpr int KPL = 8 / L2;             // second-stage DFTs per lane
-    // Transpose regions per (aperture, row, half): 8 rows k1 x L2 columns, each
-    // row padded by one float2 so that the stores of one k1 and the loads of
-    // one column are free of bank conflicts.
-    static constexpr bool V4 = NX == 128;          // second-stage reads as float4 pairs
-    static constexpr int TS = V4 ? L2 + 2 : L2 + 1;   // transpose row (float2)
-    static constexpr int RS = V4 ? 8 * TS + 8 : 8 * TS;   // transpose region (float2), 16 mod 32 words
-    static __device__ __forceinline__ int tpos(int k1, int col) { return k1 * TS + col; }
+    // Transpose regions per (aperture, row, half): 8 rows k1 x L2 columns of
+    // float2, stored 8 bytes a lane (16 lanes at a time) and read back as float4
+    // pairs (8 lanes at a time). Row stride TS and region stride RS keep both free
+    // of bank conflicts over the regions that lanes at work together touch:
+    //   nx 128: 2 regions per store, 1 per load; rows padded to TS = 10, RS = 16 mod 32 words
+    //   nx 64: 4 and 2 regions; TS = 4 with the halves of rows 4-7 swapped, RS = 8 mod 32 words
+    //   nx 32: 8 and 4 regions; TS = 2, RS = 4 mod 32 words
+    //   nx 16: the half transform is the first factor alone; nothing is transposed
+    // (with rows padded by one float2 and regions 0 or 16 words apart, as suits nx
+    // 128, the lanes of 2 to 16 regions met in one bank: a bin of nx = 16 took 13 us
+    // of a CTA, nx = 32 and 64 4- and 2-way conflicts).
+    static constexpr int TS = NX == 128 ? L2 + 2 : L2;
+    static constexpr int RS = NX == 128 ? 8 * TS + 8 : NX == 64 ? 36 : NX == 32 ? 18 : 0;
+    static __device__ __forceinline__ int tpos(int k1, int col)
+    {
+        return k1 * TS + (NX == 64 ? col ^ ((k1 >> 2) << 1) : col);
+    }
     static_assert(NX == 16 || NX == 32 || NX == 64 || NX == 128, "built lateral lengths");
 };
 
@@ -158,11 +168,14 @@ constexpr size_t prop_smem_bytes()
 {
     using S = Shape<NX, RPL>;
     constexpr int NSTAGE = prop_nstage(RPL, NX);
+    // the transposes; the cluster reduction of prop_corr_kernel keeps a tile's sums there
+    constexpr size_t transposes = (size_t)prop_warps(RPL, NX) * NAP * S::RPW * 2 * S::RS * sizeof(float2);
+    constexpr size_t sums = RPL == 1 ? (size_t)Acc<NAP>::N * S::RPC * NX * sizeof(float) : 0;
     return (size_t)128                                    // full / empty mbarriers
            + (size_t)NSTAGE * 2 * NAP * NX * sizeof(float2)   // paired spectra, one per stage
            + (size_t)NSTAGE * NX * sizeof(uint4)          // phase words + evanescent coefficients
            + (size_t)(NX / 2) * sizeof(float2)            // exp(+2 pi i m / (nx/2))
-           + (size_t)prop_warps(RPL, NX) * NAP * S::RPW * 2 * S::RS * sizeof(float2);  // transposes
+           + (transposes > sums ? transposes : sums);
 }
 
 // Eq. 4 (with the Appendix A completion) for one pixel and one pair:
@@ -450,8 +463,10 @@ __device__ __forceinline__ bool prop_bins(const PropSmem<NAP, NX, RPL> &sm, cons
         while (issued < nb && issued < NSTAGE - 1) issue_next();
 
     float2 twk[8];     // the lane's second-factor twiddles, for every bin
+    if constexpr (L2 > 1) {
 #pragma unroll
-    for (int k1 = 1; k1 < 8; ++k1) twk[k1] = sW[(n2 * k1) & (H - 1)];
+        for (int k1 = 1; k1 < 8; ++k1) twk[k1] = sW[(n2 * k1) & (H - 1)];
+    }
     int done = 0;      // bins this warp has finished
     for (int i = 0; i < nb; ++i) {
         if (tid == 0 && issued < nb) ok = issue_next();
@@ -503,7 +518,9 @@ __device__ __forceinline__ bool prop_bins(const PropSmem<NAP, NX, RPL> &sm, cons
         // first factor: 8-point DFT over n1, twiddle, into the transpose region.
         // The lane's twiddles are loaded once for all apertures (the compiler
         // reloads them per aperture otherwise; measured 2% faster). One spectra
-        // load serves the lane's RPL rows.
+        // load serves the lane's RPL rows. With one column (nx = 16) the factor is
+        // the whole half transform and stays in registers.
+        float2 px[L2 == 1 ? RPL : 1][L2 == 1 ? NAP : 1][8];
 #pragma unroll
         for (int q = 0; q < NAP; ++q) {
             float2 x[RPL][8];
@@ -523,13 +540,18 @@ __device__ __forceinline__ bool prop_bins(const PropSmem<NAP, NX, RPL> &sm, cons
 #pragma unroll
             for (int rr = 0; rr < RPL; ++rr) {
                 IDft<8>::run(x[rr]);
-                float2 *reg = myT + ((q * RPW + r * RPL + rr) * 2 + g) * RS;
+                if constexpr (L2 == 1) {
 #pragma unroll
-                for (int k1 = 0; k1 < 8; ++k1)
-                    reg[S::tpos(k1, n2)] = k1 ? cmul(x[rr][k1], twk[k1]) : x[rr][k1];
+                    for (int k1 = 0; k1 < 8; ++k1) px[rr][q][k1] = x[rr][k1];
+                } else {
+                    float2 *reg = myT + ((q * RPW + r * RPL + rr) * 2 + g) * RS;
+#pragma unroll
+                    for (int k1 = 0; k1 < 8; ++k1)
+                        reg[S::tpos(k1, n2)] = k1 ? cmul(x[rr][k1], twk[k1]) : x[rr][k1];
+                }
             }
         }
-        __syncwarp();
+        if constexpr (L2 > 1) __syncwarp();
 
         // second factor: L2-point DFTs over n2; lane owns pixels i = 2(k1 + 8 k2) + g
 #pragma unroll
@@ -538,26 +560,25 @@ __device__ __forceinline__ bool prop_bins(const PropSmem<NAP, NX, RPL> &sm, cons
             float2 p[NAP][NOUT];
 #pragma unroll
             for (int q = 0; q < NAP; ++q) {
-                const float2 *reg = myT + ((q * RPW + r * RPL + rr) * 2 + g) * RS;
+                if constexpr (L2 == 1) {
 #pragma unroll
-                for (int s = 0; s < KPL; ++s) {
-                    const int k1 = n2 * KPL + s;
-                    float2 v[L2];
-                    if constexpr (S::V4) {
-                        const float4 *reg4 = reinterpret_cast<const float4 *>(reg + k1 * S::TS);
+                    for (int k1 = 0; k1 < 8; ++k1) p[q][k1] = px[rr][q][k1];
+                } else {
+                    const float2 *reg = myT + ((q * RPW + r * RPL + rr) * 2 + g) * RS;
+#pragma unroll
+                    for (int s = 0; s < KPL; ++s) {
+                        const int k1 = n2 * KPL + s;
+                        float2 v[L2];
 #pragma unroll
                         for (int t = 0; t < L2; t += 2) {
-                            const float4 w4 = reg4[t / 2];
+                            const float4 w4 = *reinterpret_cast<const float4 *>(reg + S::tpos(k1, t));
                             v[t] = make_float2(w4.x, w4.y);
                             v[t + 1] = make_float2(w4.z, w4.w);
                         }
-                    } else {
+                        IDft<L2>::run(v);
 #pragma unroll
-                        for (int t = 0; t < L2; ++t) v[t] = reg[S::tpos(k1, t)];
+                        for (int k2 = 0; k2 < L2; ++k2) p[q][s * L2 + k2] = v[k2];
                     }
-                    IDft<L2>::run(v);
-#pragma unroll
-                    for (int k2 = 0; k2 < L2; ++k2) p[q][s * L2 + k2] = v[k2];
                 }
             }
 
