@@ -41,7 +41,7 @@ __device__ uint64_t turns_to_word(double turns)
 __global__ void tables_kernel(const int *__restrict__ bins, int n_bins, int nx, int nt, double fs,
                               double c, double pitch, double z0, double dz, int evanescent_zero,
                               uint4 *__restrict__ phase, float *__restrict__ live, int *__restrict__ bin_evan,
-                              float2 *__restrict__ tw_t, float2 *__restrict__ tw_x)
+                              float2 *__restrict__ tw_t, int stage_m, float2 *__restrict__ tw_x)
 {
     const double two_pi = 6.283185307179586476925286766559;
     int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -68,8 +68,25 @@ __global__ void tables_kernel(const int *__restrict__ bins, int n_bins, int nx, 
         phase[idx] = w;
     }
     if (idx < nt) {
+        int m = idx;
+        if (stage_m > 0 && idx >= stage_m) {
+            // second half of a power-of-2 plan's table: the twiddles exp(-2 pi i m / M),
+            // M = stage_m = nt / 2, in the order the radix-8 stages of the time FFT read them
+            const int M = stage_m;
+            int i = idx - M, Ns = 1;
+            m = 0;
+            while (Ns < M) {
+                const int R = 8 * Ns <= M ? 8 : 4 * Ns <= M ? 4 : 2, cnt = Ns > 1 ? (R - 1) * Ns : 0;
+                if (i < cnt) {
+                    m = 2 * ((i / Ns + 1) * (i % Ns) * (M / (R * Ns)));
+                    break;
+                }
+                i -= cnt;
+                Ns *= R;
+            }
+        }
         double s, co;
-        sincospi(-2.0 * (double)idx / (double)nt, &s, &co);
+        sincospi(-2.0 * (double)m / (double)nt, &s, &co);
         tw_t[idx] = make_float2((float)co, (float)s);
     }
     if (idx < nx) {
@@ -112,79 +129,109 @@ __device__ __forceinline__ void fdft8(float2 (&v)[8])
     }
 }
 
-// Forward FFTs (exp(-2 pi i m / n)) of `batch` contiguous n-point sequences in
-// shared memory. With MAXR = 8: radix-8 stages while they fit, then radix-4;
-// with MAXR = 4: radix-4 stages. Then one radix-2 stage if a factor 2 is left.
-// Auto-sort ordering (a stage of radix R takes sub-transforms of length Ns to
-// R Ns), so the output is in natural order. tw[m] holds exp(-2 pi i m / n)
-// for m < n. x and y are ping-pong buffers; the return value is the buffer
-// with the result. Every thread of the CTA must call it.
+// Shared-memory index of element i of a sequence: one float2 of padding after
+// every 16 (128 bytes), so that the strided writes of a first stage fall into
+// different banks. A sequence takes fft_len(n) entries.
+__host__ __device__ __forceinline__ constexpr int fpad(int i) { return i + (i >> 4); }
+__host__ __device__ constexpr int fft_len(int n) { return fpad(n); }
+
+// Twiddles of every stage after the first, in the order the stages read them:
+// for a radix-R stage that takes sub-transforms of length Ns to R Ns, entries
+// [(r - 1) Ns + k] = exp(-2 pi i r k / (R Ns)), r = 1 .. R - 1, k < Ns, so that
+// consecutive threads read consecutive entries. tw(m) gives exp(-2 pi i m / n).
+// Fewer than n entries in all.
+template <int MAXR, class F>
+__device__ void stage_twiddles(float2 *dst, int n, int tid, int nth, F tw)
+{
+    int Ns = 1;
+    while (Ns < n) {
+        const int R = MAXR == 8 && 8 * Ns <= n ? 8 : 4 * Ns <= n ? 4 : 2;
+        if (Ns > 1) {
+            const int ts = n / (R * Ns), ln = 31 - __clz(Ns);
+            for (int i = tid; i < (R - 1) * Ns; i += nth) dst[i] = tw(((i >> ln) + 1) * (i & (Ns - 1)) * ts);
+            dst += (R - 1) * Ns;
+        }
+        Ns *= R;
+    }
+}
+
+// Forward FFTs (exp(-2 pi i m / n)) of `batch` n-point sequences in shared
+// memory, fft_len(n) entries apart (element i at fpad(i)). With MAXR = 8: radix-8
+// stages while they fit, then radix-4; with MAXR = 4: radix-4 stages. Then one
+// radix-2 stage if a factor 2 is left. Auto-sort ordering (a stage of radix R
+// takes sub-transforms of length Ns to R Ns), so the output is in natural order.
+// tw: stage_twiddles. x and y are ping-pong buffers; the return value is the
+// buffer with the result. Every thread of the CTA must call it.
+// Bound by shared memory: a stage reads and writes every element once. Unpadded,
+// with the twiddles read from one table of n entries, two thirds of the
+// wavefronts were bank conflicts (4,276 a 4096-sample channel, 85% of the pipe).
 template <int MAXR>
 __device__ float2 *stockham(float2 *x, float2 *y, int n, int log2n, int batch, const float2 *tw, int tid, int nth)
 {
+    const int len = fft_len(n);
     int Ns = 1;
     if constexpr (MAXR == 8) {
         const int q8 = n >> 3;
         const int lq8 = log2n - 3;
         for (; 8 * Ns <= n; Ns <<= 3) {
-            const int ts = n / (8 * Ns);
             for (int t = tid; t < batch * q8; t += nth) {
                 const int bt = t >> lq8, j = t & (q8 - 1);
-                const float2 *xb = x + bt * n;
-                float2 *yb = y + bt * n;
+                const float2 *xb = x + bt * len;
+                float2 *yb = y + bt * len;
                 const int k = j & (Ns - 1);
                 float2 v[8];
 #pragma unroll
-                for (int r = 0; r < 8; ++r) v[r] = xb[j + r * q8];
+                for (int r = 0; r < 8; ++r) v[r] = xb[fpad(j + r * q8)];
                 if (Ns > 1) {
 #pragma unroll
-                    for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], tw[r * k * ts]);
+                    for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], tw[(r - 1) * Ns + k]);
                 }
                 fdft8(v);
                 const int base = (j - k) * 8 + k;
 #pragma unroll
-                for (int r = 0; r < 8; ++r) yb[base + r * Ns] = v[r];
+                for (int r = 0; r < 8; ++r) yb[fpad(base + r * Ns)] = v[r];
             }
             __syncthreads();
+            if (Ns > 1) tw += 7 * Ns;
             float2 *tmp = x; x = y; y = tmp;
         }
     }
     const int q4 = n >> 2;
     const int lq4 = log2n - 2;
     for (; 4 * Ns <= n; Ns <<= 2) {
-        const int ts = n / (4 * Ns);
         for (int t = tid; t < batch * q4; t += nth) {
             const int bt = t >> lq4, j = t & (q4 - 1);
-            const float2 *xb = x + bt * n;
-            float2 *yb = y + bt * n;
+            const float2 *xb = x + bt * len;
+            float2 *yb = y + bt * len;
             const int k = j & (Ns - 1);
-            float2 v0 = xb[j], v1 = xb[j + q4], v2 = xb[j + 2 * q4], v3 = xb[j + 3 * q4];
+            float2 v0 = xb[fpad(j)], v1 = xb[fpad(j + q4)], v2 = xb[fpad(j + 2 * q4)], v3 = xb[fpad(j + 3 * q4)];
             if (Ns > 1) {
-                v1 = cmul(v1, tw[k * ts]);
-                v2 = cmul(v2, tw[2 * k * ts]);
-                v3 = cmul(v3, tw[3 * k * ts]);
+                v1 = cmul(v1, tw[k]);
+                v2 = cmul(v2, tw[Ns + k]);
+                v3 = cmul(v3, tw[2 * Ns + k]);
             }
             float2 s02 = cadd(v0, v2), d02 = csub(v0, v2);
             float2 s13 = cadd(v1, v3), d13 = csub(v1, v3);
             float2 md13 = make_float2(d13.y, -d13.x);   // -i * d13
             const int base = (j - k) * 4 + k;
-            yb[base] = cadd(s02, s13);
-            yb[base + Ns] = cadd(d02, md13);
-            yb[base + 2 * Ns] = csub(s02, s13);
-            yb[base + 3 * Ns] = csub(d02, md13);
+            yb[fpad(base)] = cadd(s02, s13);
+            yb[fpad(base + Ns)] = cadd(d02, md13);
+            yb[fpad(base + 2 * Ns)] = csub(s02, s13);
+            yb[fpad(base + 3 * Ns)] = csub(d02, md13);
         }
         __syncthreads();
+        if (Ns > 1) tw += 3 * Ns;
         float2 *tmp = x; x = y; y = tmp;
     }
     if (Ns < n) {  // radix-2 stage with Ns = n/2
         const int h = n >> 1;
         for (int t = tid; t < batch * h; t += nth) {
             const int bt = t >> (log2n - 1), j = t & (h - 1);
-            const float2 *xb = x + bt * n;
-            float2 *yb = y + bt * n;
-            float2 v0 = xb[j], v1 = cmul(xb[j + h], tw[j]);
-            yb[j] = cadd(v0, v1);
-            yb[j + h] = csub(v0, v1);
+            const float2 *xb = x + bt * len;
+            float2 *yb = y + bt * len;
+            float2 v0 = xb[fpad(j)], v1 = cmul(xb[fpad(j + h)], tw[j]);
+            yb[fpad(j)] = cadd(v0, v1);
+            yb[fpad(j + h)] = csub(v0, v1);
         }
         __syncthreads();
         x = y;
@@ -211,20 +258,33 @@ time_fft_kernel(const float *__restrict__ rf, int ne, int nt, int log2nt, const 
 {
     extern __shared__ __align__(16) float2 sbuf[];
     const int M = nt >> 1;
-    float2 *x = sbuf, *y = sbuf + M, *tws = sbuf + 2 * M;
+    float2 *x = sbuf, *y = sbuf + fft_len(M), *tws = sbuf + 2 * fft_len(M);
     const int f = blockIdx.y, e = blockIdx.x;
     const float4 *src = reinterpret_cast<const float4 *>(rf + ((size_t)f * ne + e) * nt);
-    float4 *x4 = reinterpret_cast<float4 *>(x);
-    for (int m = threadIdx.x; m < M; m += TFFT_THREADS) tws[m] = tw[2 * m];    // exp(-2 pi i m / M), a plan table
+    // twiddles from the plan's table: its second half holds the radix-8 stages',
+    // its first half exp(-2 pi i k / nt), from which radix 4 gathers (half a turn on,
+    // the sign changes)
+    if constexpr (MAXR == 8) {
+        for (int i = threadIdx.x; i < M; i += TFFT_THREADS) tws[i] = tw[M + i];
+    } else {
+        stage_twiddles<MAXR>(tws, M, threadIdx.x, TFFT_THREADS, [&](int m) {
+            const float2 w = tw[2 * m < M ? 2 * m : 2 * m - M];
+            return 2 * m < M ? w : make_float2(-w.x, -w.y);
+        });
+    }
     ptx::pdl_wait();
     if (e == 0 && threadIdx.x == 0) fmax[f] = 0u;
-    for (int i = threadIdx.x; i < nt / 4; i += TFFT_THREADS) x4[i] = src[i];  // (x0,x1),(x2,x3) pairs
+    for (int i = threadIdx.x; i < nt / 4; i += TFFT_THREADS) {   // (x0,x1),(x2,x3) pairs
+        const float4 v = src[i];
+        x[fpad(2 * i)] = make_float2(v.x, v.y);
+        x[fpad(2 * i + 1)] = make_float2(v.z, v.w);
+    }
     __syncthreads();
     float2 *Z = stockham<MAXR>(x, y, M, log2nt - 1, 1, tws, threadIdx.x, TFFT_THREADS);
     ptx::pdl_trigger();
     for (int b = threadIdx.x; b < n_bins; b += TFFT_THREADS) {
         const int k = bins[b];                                 // 0 < k < M
-        const float2 zk = Z[k], zm = Z[M - k];
+        const float2 zk = Z[fpad(k)], zm = Z[fpad(M - k)];
         const float2 E = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
         const float2 O = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
         S[((size_t)f * n_bins + b) * nev + (size_t)e * cstep] = cadd(E, cmul(tw[k], O));
@@ -255,16 +315,17 @@ lateral_kernel(const float2 *__restrict__ S, int ne, int nx, int log2nx, int n_b
                size_t live_fs, float2 *__restrict__ Q)
 {
     extern __shared__ __align__(16) float2 lbuf[];
-    float2 *x = lbuf, *y = lbuf + napq * nx, *tws = lbuf + 2 * napq * nx;
+    const int len = fft_len(nx);
+    float2 *x = lbuf, *y = lbuf + napq * len, *tws = lbuf + 2 * napq * len;
     const int f = blockIdx.y, b = blockIdx.x;
     const float2 *s = S + ((size_t)f * n_bins + b) * ne;
-    for (int i = threadIdx.x; i < nx; i += LAT_THREADS) tws[i] = twx[i];   // a plan table
+    stage_twiddles<4>(tws, nx, threadIdx.x, LAT_THREADS, [&](int m) { return twx[m]; });   // from a plan table
     ptx::pdl_wait();
     for (int i = threadIdx.x; i < napq * nx; i += LAT_THREADS) {
         const int q = i / nx, e = i - q * nx;
         const float2 v = s[e];
         const float a = apod[q * ne + e];
-        x[i] = make_float2(a * v.x, a * v.y);
+        x[q * len + fpad(e)] = make_float2(a * v.x, a * v.y);
     }
     __syncthreads();
     const float2 *X = stockham<4>(x, y, nx, log2nx, napq, tws, threadIdx.x, LAT_THREADS);
@@ -275,10 +336,10 @@ lateral_kernel(const float2 *__restrict__ S, int ne, int nx, int log2nx, int n_b
     for (int i = threadIdx.x; i < napq * nx; i += LAT_THREADS) {
         const int q = i / nx, u = i & (nx - 1);
         const float l = live[(size_t)f * live_fs + (size_t)b * nx + u] * inv_nx;
-        const float2 v = make_float2(X[i].x * l, X[i].y * l);
+        const float2 t = X[q * len + fpad(u)], v = make_float2(t.x * l, t.y * l);
         const int hi = u >= H ? 1 : 0, u0 = u - hi * H, n1 = u0 / L2, n2 = u0 - n1 * L2;
-        float ws, wc;
-        sincospif(2.0f * (float)u0 / (float)nx, &ws, &wc);   // W^u0, exact argument
+        const float2 w = twx[u0];                            // W^u0 is its conjugate
+        const float wc = w.x, ws = -w.y;
         const float sg = hi ? -1.0f : 1.0f;
         const float2 vw = make_float2(sg * (wc * v.x - ws * v.y), sg * (wc * v.y + ws * v.x));
         const size_t base = (size_t)(q * 8 + n1) * 2;
@@ -294,9 +355,9 @@ int ilog2i(int v)
     return l;
 }
 
-size_t time_fft_smem(int nt) { return (size_t)3 * (nt / 2) * sizeof(float2); }
+size_t time_fft_smem(int nt) { return ((size_t)2 * fft_len(nt / 2) + nt / 2) * sizeof(float2); }
 
-size_t lateral_smem(int nx, int napq) { return ((size_t)2 * napq * nx + nx) * sizeof(float2); }
+size_t lateral_smem(int nx, int napq) { return ((size_t)2 * napq * fft_len(nx) + nx) * sizeof(float2); }
 
 }  // namespace
 
@@ -309,7 +370,7 @@ cudaError_t launch_tables(const pam_plan_s &p, cudaStream_t st)
     int blocks = (n + 255) / 256;
     tables_kernel<<<blocks, 256, 0, st>>>(p.t.bins, p.n_bins, p.nx, p.nt, p.d.fs_hz, p.d.c_mps, p.pitch_x,
                                           p.d.z0_m, p.d.dz_m, (p.d.flags & PAM_EVANESCENT_ZERO) ? 1 : 0,
-                                          p.t.phase, p.t.live, p.t.bin_evan, p.t.tw_t, p.t.tw_x);
+                                          p.t.phase, p.t.live, p.t.bin_evan, p.t.tw_t, p.nt / 2, p.t.tw_x);
     return cudaGetLastError();
 }
 
@@ -346,7 +407,7 @@ cudaError_t launch_tables_frame(const pam_plan_s &p, const int *bins, int n_bins
     if (nt > n) n = nt;
     tables_kernel<<<(n + 255) / 256, 256, 0, st>>>(bins, n_bins, p.nx, nt, p.d.fs_hz, p.d.c_mps, p.pitch_x,
                                                     p.d.z0_m, p.d.dz_m, (p.d.flags & PAM_EVANESCENT_ZERO) ? 1 : 0,
-                                                    phase, live, bin_evan, tw_t, p.t.tw_x);
+                                                    phase, live, bin_evan, tw_t, 0, p.t.tw_x);
     return cudaGetLastError();
 }
 

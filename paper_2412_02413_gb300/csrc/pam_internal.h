@@ -94,7 +94,9 @@ struct Tables {
     int *bins = nullptr;          // [n_bins]
     float *apod = nullptr;        // [n_apod][n_elem]
     float *ones = nullptr;        // [n_elem]
-    float2 *tw_t = nullptr;       // [nt]   exp(-2 pi i m / nt)
+    // [nt] exp(-2 pi i m / nt), m < nt/2; then the twiddles of the time FFT's radix-8 stages in
+    // their order (batches, with tables of their own: exp(-2 pi i m / nt) throughout)
+    float2 *tw_t = nullptr;
     float2 *tw_x = nullptr;       // [nx]   exp(-2 pi i m / nx)
     // [n_bins][nx] per lateral bin u: {anchor_hi, step_hi, step_lo, ecoef bits}. The phase of row j,
     // in turns * 2^32, is anchor_hi + j*step_hi + hi32(j*step_lo) (mod 2^32): the top word of the
