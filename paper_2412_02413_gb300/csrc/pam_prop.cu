@@ -855,19 +855,22 @@ epi_reduce_kernel(const float4 *__restrict__ part, int n_split, int npix4, int n
 // more CTAs share, its slots added in CTA order (deterministic), then the
 // per-pixel epilogue. A tile inside one CTA's share was finished by that CTA;
 // its blocks return at once (a block's 128 pixels never straddle tiles).
-// One warp per accumulator adds 32 groups of four pixels; then four warps (of AS:
-// one) finish a pixel per thread. Bound by the latency of the slots' loads (L2)
-// and of the square roots, divisions and the cube root behind them.
-template <int NAP>
-__global__ void __launch_bounds__(Acc<NAP>::N < 4 ? 128 : 32 * Acc<NAP>::N)
+// RED_G warps per accumulator each add a share of the slots for 32 groups of four
+// pixels; the shares are added in order and four warps finish a pixel per thread.
+// Bound by the latency of the slots' loads (L2) and of the square roots, divisions
+// and the cube root behind them. RED_G = 4 while its blocks fit the SMs at once, two
+// to an SM (a 64 x 128 frame, 76 slots a pixel: 7.3 us against 9.5 us with one
+// warp per accumulator), else 2 (a 128 x 512 frame, 15 slots: 7.0 us with 2, 9.1
+// with 4, 7.8 with one, which took 10 us while one warp of six did the pixel math).
+template <int NAP, int RED_G>
+__global__ void __launch_bounds__(32 * RED_G * Acc<NAP>::N, NAP == 3 ? 8 / RED_G : 4)
 epi_reduce_seg_kernel(const float4 *__restrict__ part, int npix4, int nx, int rpc, int n_bins, int tiles, long long W,
                       int G, EpiOut out)
 {
-    constexpr int NACC = Acc<NAP>::N, NT = NACC < 4 ? 128 : 32 * NACC;
-    __shared__ float4 sA[NACC][32];
-    __shared__ float wmax[NT / 32];
+    constexpr int NACC = Acc<NAP>::N;
+    __shared__ float4 sA[RED_G][NACC][32];
     const int f = blockIdx.y;
-    const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int c = (threadIdx.x >> 5) % NACC, sg = (threadIdx.x >> 5) / NACC, lane = threadIdx.x & 31;
     const int tile4 = rpc * nx / 4;                    // float4 groups per tile
     const int tile = (blockIdx.x * 32) / tile4;
     const long long tt = (long long)f * tiles + tile;
@@ -878,42 +881,54 @@ epi_reduce_seg_kernel(const float4 *__restrict__ part, int npix4, int nx, int rp
     pdl_wait();
     if (cf == cl) return;                              // block-uniform
     const int x4 = blockIdx.x * 32 + lane;
-    if (c < NACC) {
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (x4 < npix4) {
-            // The slots' loads are all issued before the sums (in CTA order), in
-            // batches of 16, so that their latencies overlap.
-            constexpr int MAXS = 16;
-            const size_t off = (size_t)c * tile4 + (x4 - tile * tile4);
-            const int ns = cl - cf + 1;
-            for (int base = 0; base < ns; base += MAXS) {
-                float4 v[MAXS];
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (x4 < npix4) {
+        // the loads of up to MAXS slots are issued before their sums (in CTA order)
+        constexpr int MAXS = 4;
+        const size_t off = (size_t)c * tile4 + (x4 - tile * tile4);
+        const int ns = cl - cf + 1, s1 = ns * (sg + 1) / RED_G;
+        for (int base = ns * sg / RED_G; base < s1; base += MAXS) {
+            float4 v[MAXS];
 #pragma unroll
-                for (int k = 0; k < MAXS; ++k) {
-                    const int cc = cf + base + k;
-                    const size_t slot = cc == cf ? (size_t)cf_slot : 2 * (size_t)cc;
-                    if (base + k < ns) v[k] = part[slot * NACC * tile4 + off];
-                }
-#pragma unroll
-                for (int k = 0; k < MAXS; ++k)
-                    if (base + k < ns) {
-                        a.x += v[k].x; a.y += v[k].y; a.z += v[k].z; a.w += v[k].w;
-                    }
+            for (int k = 0; k < MAXS; ++k) {
+                const int cc = cf + base + k;
+                const size_t slot = cc == cf ? (size_t)cf_slot : 2 * (size_t)cc;
+                if (base + k < s1) v[k] = part[slot * NACC * tile4 + off];
             }
+#pragma unroll
+            for (int k = 0; k < MAXS; ++k)
+                if (base + k < s1) {
+                    a.x += v[k].x; a.y += v[k].y; a.z += v[k].z; a.w += v[k].w;
+                }
         }
-        sA[c][lane] = a;
     }
+    sA[sg][c][lane] = a;
     pdl_trigger();
     __syncthreads();
     float rmax = 0.0f;
-    const int x = 128 * blockIdx.x + threadIdx.x;      // pixel of the full-width row grid
-    if (threadIdx.x < 128 && x < 4 * npix4) {
+    constexpr int NT = 32 * RED_G * NACC;
+#pragma unroll
+    for (int i = threadIdx.x; i < 128; i += NT) {
+        const int x = 128 * blockIdx.x + i;            // pixel of the full-width row grid
+        if (x >= 4 * npix4) break;
         float acc[NACC];
 #pragma unroll
-        for (int k = 0; k < NACC; ++k) acc[k] = reinterpret_cast<const float *>(&sA[k][0])[threadIdx.x];
-        rmax = pixel_epilogue<NAP>(acc, out, (size_t)f * out.npix, x / nx, x % nx);
+        for (int k = 0; k < NACC; ++k) {
+            float v = reinterpret_cast<const float *>(&sA[0][k][0])[i];
+#pragma unroll
+            for (int g = 1; g < RED_G; ++g) v += reinterpret_cast<const float *>(&sA[g][k][0])[i];
+            acc[k] = v;
+        }
+        rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc, out, (size_t)f * out.npix, x / nx, x % nx));
     }
-    if constexpr (NAP > 1) block_max_to(rmax, out.fmax + f, wmax, NT);
+    if constexpr (NAP > 1) {
+        // the largest rho of the 128 pixels, folded into the frame's maximum (rho > 0)
+        if (threadIdx.x < 128) {
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, d));
+            if (lane == 0) atomicMax(out.fmax + f, __float_as_uint(rmax));
+        }
+    }
 }
 
 // rho_n = rho / max (Sec. II-A: the maximum becomes exactly 1) and the image
@@ -1373,8 +1388,11 @@ cudaError_t launch_epilogue(const pam_plan_s &p, int n_frames, int napq, int n_s
         const int G = prop_seg_ctas(p, n_frames);
         const float4 *part = reinterpret_cast<const float4 *>(p.w.part);
         dim3 rgrid((npix4 + 31) / 32, n_frames);
-        auto reduce = napq == 1 ? epi_reduce_seg_kernel<1> : napq == 2 ? epi_reduce_seg_kernel<2> : epi_reduce_seg_kernel<3>;
-        cudaError_t e = launch_pdl(p.pdl, reduce, rgrid, napq == 3 ? 32 * Acc<3>::N : 128, 0, st, part, npix4, p.nx, rows,
+        const int rg = (long long)rgrid.x * rgrid.y <= 2LL * p.num_sms ? 4 : 2;
+        auto reduce = napq == 1 ? (rg == 4 ? epi_reduce_seg_kernel<1, 4> : epi_reduce_seg_kernel<1, 2>)
+                      : napq == 2 ? (rg == 4 ? epi_reduce_seg_kernel<2, 4> : epi_reduce_seg_kernel<2, 2>)
+                                  : (rg == 4 ? epi_reduce_seg_kernel<3, 4> : epi_reduce_seg_kernel<3, 2>);
+        cudaError_t e = launch_pdl(p.pdl, reduce, rgrid, 32 * rg * n_acc(napq), 0, st, part, npix4, p.nx, rows,
                                    p.n_bins, tiles, W, G, out);
         if (e != cudaSuccess) return e;
     } else if (from_partials || !prop_uses_cluster(n_split)) {
