@@ -265,6 +265,18 @@ size_t gemm_smem(int K, bool split, bool pair, int fg)
     return gemm_stages(K, split, pair, fg) * gemm_stage_bytes(K, split ? 2 : 1, pair, fg) + GEMM_SMEM_EXTRA;
 }
 
+// Band form: start, in the (frame group, row, bin) sequence, of CTA c's share when G
+// CTAs take equal contiguous shares of whole bands. One CTA per (row, group) left
+// the last wave partly empty (32 frames of 512 rows on 152 SMs: 4 waves for 3.4,
+// 930 us; a band at a time 836). The other forms keep one CTA per (row, group): their
+// rows cannot be split without changing the order of the sums, and running rows on in
+// one CTA costs the fold registers (960 us for 21 BF16 frames against 830).
+__host__ __device__ __forceinline__ long long band_share(int rows, int groups, int c, int G, int n_bins, int n_bands)
+{
+    const long long w = (long long)rows * groups * n_bands * c / G, u = w / n_bands;
+    return u * n_bins + (long long)n_bins * (w - u * n_bands) / n_bands;
+}
+
 // steps: element block of K step st in bits 4 (st % 16) of steps[st / 16].
 // BANDS: instead of the per-aperture sums, fold the full-aperture energy
 // |p_1 + p_2 + p_3|^2 (Eq. 3 with apodizations that sum to one) and write it
@@ -281,7 +293,8 @@ template <int NAP, bool FP16, bool SPLIT, bool BANDS = false, bool PAIR = false,
 __global__ void __launch_bounds__(gemm_threads<NAP>(), 1)
 prec_gemm_kernel(const uint32_t *__restrict__ chi, const uint32_t *__restrict__ clo, const uint8_t *__restrict__ Bhi,
                  const uint8_t *__restrict__ Blo, ulonglong2 steps, int4 kq, int n_bins, int nz, int F, int NST,
-                 const unsigned *__restrict__ smax, float *__restrict__ part, int *__restrict__ status, int n_bands)
+                 const unsigned *__restrict__ smax, float *__restrict__ part, int *__restrict__ status, int n_bands,
+                 int groups)
 {
     static_assert(!BANDS || NAP == 3, "band energies fold three apertures");
     static_assert(!(BANDS && PAIR), "the band form runs unpaired");
@@ -307,7 +320,16 @@ prec_gemm_kernel(const uint32_t *__restrict__ chi, const uint32_t *__restrict__ 
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tslot + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // Bins of this CTA, counted by i or b from 0 to n - 1: those of row j and frame group
+    // grp, or (BANDS) of its share, which starts at bin bin0 of unit u0 = group x nz + row.
     const int j = blockIdx.x, grp = blockIdx.y;
+    int n = n_bins, u0 = 0, bin0 = 0;
+    if constexpr (BANDS) {
+        const long long w0 = band_share(nz, groups, (int)blockIdx.x, (int)gridDim.x, n_bins, n_bands);
+        n = (int)(band_share(nz, groups, (int)blockIdx.x + 1, (int)gridDim.x, n_bins, n_bands) - w0);
+        u0 = (int)(w0 / n_bins);
+        bin0 = (int)(w0 - (long long)u0 * n_bins);
+    }
     const unsigned rank = PAIR ? cluster_ctarank() : 0u;
     const bool row_ok = j < nz;               // a pair's second row may lie past the grid
     const int jl = row_ok ? j : nz - 1;       // row whose c words are loaded
@@ -393,11 +415,13 @@ prec_gemm_kernel(const uint32_t *__restrict__ chi, const uint32_t *__restrict__ 
         const int s0 = (q <= 0 ? kq.x : q == 1 ? kq.y : kq.z) / 16;
         const int s1 = (q <= 0 ? kq.y : q == 1 ? kq.z : kq.w) / 16;
         int issued = 0;
+        int lu = u0, lb = bin0;   // BANDS: unit and bin of the next load
         auto load = [&](int b) {
             if (lane == 0) {
                 const int s = b % NST;
-                const size_t ob = ((size_t)grp * n_bins + b) * (PAIR ? 2 : 1) * bytesB + rank * bytesB;
-                const size_t oc = ((size_t)b * nz + jl) * NXP;
+                const int gq = BANDS ? lu / nz : grp, jq = BANDS ? lu - gq * nz : jl, bq = BANDS ? lb : b;
+                const size_t ob = ((size_t)gq * n_bins + bq) * (PAIR ? 2 : 1) * bytesB + rank * bytesB;
+                const size_t oc = ((size_t)bq * nz + jq) * NXP;
                 mbar_expect_tx(&full[s], (unsigned)(NPART * (bytesB + NXP * 4)));
                 bulk_g2s(sB(s), Bhi + ob, (unsigned)bytesB, &full[s]);
                 bulk_g2s(sC(s), chi + oc, NXP * 4, &full[s]);
@@ -408,18 +432,24 @@ prec_gemm_kernel(const uint32_t *__restrict__ chi, const uint32_t *__restrict__ 
             }
             __syncwarp();
             issued = b + 1;
+            if constexpr (BANDS) {
+                if (++lb == n_bins) {
+                    lb = 0;
+                    ++lu;
+                }
+            }
         };
         if (producer)
-            for (int b = 0; b < n_bins && b < NST; ++b) load(b);
+            for (int b = 0; b < n && b < NST; ++b) load(b);
         bool ok = true, any = false;
         if (producer) {
-            for (int b = NST; b < n_bins && ok; ++b) {
+            for (int b = NST; b < n && ok; ++b) {
                 // stage of bin b - NST is free once every aperture's MMAs of that bin are done
                 ok = __all_sync(0xffffffffu, wait(&sfree[b % NST], (unsigned)(b / NST - 1) & 1u));
                 if (ok) load(b);
             }
         } else if (!PAIR || rank == 0) {   // a pair's MMAs are issued by its rank-0 CTA
-            for (int b = 0; b < n_bins && ok; ++b) {
+            for (int b = 0; b < n && ok; ++b) {
                 const int s = b % NST, t = b & 1;
                 // go[t]: the blocks of bin b are built (which the build warps did after
                 // its copy landed) and accumulator set t was read out for bin b - 2
@@ -586,30 +616,38 @@ prec_gemm_kernel(const uint32_t *__restrict__ chi, const uint32_t *__restrict__ 
         // the stage of bin b+2-NST (NST >= 2), whose MMAs are done once fold(b)
         // has seen bin b's accumulators.
         const size_t npix = (size_t)nz * NXP;
-        int band = 0;
+        int unit = u0, bin = bin0, band = 0;   // BANDS: of the bin being folded
+        if constexpr (BANDS)
+            while ((int)(((long long)n_bins * (band + 1)) / n_bands) <= bin0) ++band;
         // write the band sums of this warp's frames and restart them
         auto flush = [&]() {
+            const int gq = unit / nz, jq = unit - gq * nz;
 #pragma unroll
             for (int f = 0; f < FW; ++f) {
-                const int fr = grp * FG + fh * FW + f;
+                const int fr = gq * FG + fh * FW + f;
                 if (fr < F) {
                     const float s2 = ldexpf(1.0f, 2 * frame_exp(smax[fr]));
                     const float v = (f & 1) ? acc[f >> 1][0].y : acc[f >> 1][0].x;
-                    part[((size_t)fr * n_bands + band) * npix + (size_t)j * NXP + i_epi] = v * s2;
+                    part[((size_t)fr * n_bands + band) * npix + (size_t)jq * NXP + i_epi] = v * s2;
                 }
             }
 #pragma unroll
             for (int f = 0; f < FW / 2; ++f) acc[f][0] = make_float2(0.f, 0.f);
         };
-        bool ok = n_bins == 0 || build(0);
-        if (ok && n_bins > 1) ok = build(1);
-        for (int b = 0; b < n_bins && ok; ++b) {
+        bool ok = n == 0 || build(0);
+        if (ok && n > 1) ok = build(1);
+        for (int b = 0; b < n && ok; ++b) {
             if (!fold(b)) ok = false;                            // tensor core: MMA(b+1)
-            if (ok && b + 2 < n_bins && !build(b + 2)) ok = false;
+            if (ok && b + 2 < n && !build(b + 2)) ok = false;
             if constexpr (BANDS) {
-                if (ok && b + 1 == (int)(((long long)n_bins * (band + 1)) / n_bands)) {
+                if (!ok) break;
+                if (++bin == (int)(((long long)n_bins * (band + 1)) / n_bands)) {
                     flush();
                     ++band;
+                }
+                if (bin == n_bins) {
+                    bin = band = 0;
+                    ++unit;
                 }
             }
         }
@@ -678,7 +716,7 @@ cudaError_t launch_gemm_t(const pam_plan_s &p, int n_frames, cudaStream_t st)
     cudaError_t e = cudaLaunchKernelEx(&cfg, prec_gemm_kernel<NAP, FP16, SPLIT, false, PAIR, FG>, p.t.c_hi, p.t.c_lo,
                                        reinterpret_cast<const uint8_t *>(p.w.Bhi),
                                        reinterpret_cast<const uint8_t *>(p.w.Blo), steps, kq, p.n_bins, p.nz, n_frames,
-                                       nst, p.w.smax, p.w.part, p.w.status, 0);
+                                       nst, p.w.smax, p.w.part, p.w.status, 0, groups);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -702,9 +740,11 @@ cudaError_t launch_bands_form(const pam_plan_s &p, const float2 *S, int n_frames
     if (gemm_stages(p.K, false, false, FG) < 2 || p.K / 16 > 32) return cudaErrorInvalidConfiguration;
     const int4 kq = make_int4(p.kq[0], p.kq[1], p.kq[2], p.kq[3]);
     const ulonglong2 steps = gemm_steps(p);
-    prec_gemm_kernel<3, FP16, false, true><<<dim3(p.nz, groups), gemm_threads<3>(), gemm_smem(p.K, false, false, FG), st>>>(
+    const long long units = (long long)p.nz * groups * n_bands;
+    const int ctas = (int)(units < p.num_sms ? units : p.num_sms);
+    prec_gemm_kernel<3, FP16, false, true><<<ctas, gemm_threads<3>(), gemm_smem(p.K, false, false, FG), st>>>(
         p.t.c_hi, nullptr, reinterpret_cast<const uint8_t *>(p.w.Bhi), nullptr, steps, kq, p.n_bins, p.nz, n_frames,
-        gemm_stages(p.K, false, false, FG), p.w.smax, bands, p.w.status, n_bands);
+        gemm_stages(p.K, false, false, FG), p.w.smax, bands, p.w.status, n_bands, groups);
     return cudaGetLastError();
 }
 
