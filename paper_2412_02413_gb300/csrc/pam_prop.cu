@@ -333,6 +333,18 @@ __device__ __forceinline__ void acc_update(unsigned tcol, const float2 (&p)[NAP]
     }
 }
 
+// Adds one bin's field of one frame to the frame's energy.
+__device__ __forceinline__ void acc_update_frame(unsigned tcol, const float2 (&p)[8])
+{
+    tmem_wait_st();   // the previous bin's stores have landed
+    float v[8];
+    tmem_ld8(tcol, v);
+    tmem_wait_ld();
+#pragma unroll
+    for (int o = 0; o < 8; ++o) v[o] = add_norm(v[o], p[o]);
+    tmem_st8(tcol, v);
+}
+
 // The sums of the thread's 8 pixels, acc[o][a], back in registers.
 template <int NAP>
 __device__ __forceinline__ void acc_read(unsigned tcol, float (&acc)[8][Acc<NAP>::N])
@@ -414,19 +426,23 @@ struct PropSmem {
 // tcol + rr * 8 * NACC. With FIELDS (one row per lane), lanes of valid rows
 // also write bin b's fields to fields_row + b * bin_stride. Returns false if a
 // bounded wait expired; the copies still in flight have landed by then.
-template <int NAP, int NX, bool FIELDS, int RPL = 1>
+// FRAMES: the NAP "apertures" are as many frames of one aperture, the first
+// `live` of them wanted: their spectra are [n_bins][1][8][2][NX/16] arrays
+// `frame_q` float2 apart, they share the phasors, and each keeps its energy
+// alone (sum q in columns tcol + 8 q).
+template <int NAP, int NX, bool FIELDS, int RPL = 1, bool FRAMES = false>
 __device__ __forceinline__ bool prop_bins(const PropSmem<NAP, NX, RPL> &sm, const float2 *__restrict__ Qf,
                                           const uint4 *__restrict__ phase, const int *__restrict__ bin_evan,
                                           int b_begin, int nb, const int (&jj)[RPL], const float (&zj)[RPL],
                                           unsigned seq, unsigned tcol, float2 *__restrict__ fields_row, bool row_ok,
-                                          size_t bin_stride)
+                                          size_t bin_stride, int live = NAP, size_t frame_q = 0)
 {
     using S = Shape<NX, RPL>;
     static_assert(!FIELDS || RPL == 1, "fields are written by the one-row form");
     constexpr int H = S::H, L2 = S::L2, LPR = S::LPR, RPW = S::RPW, KPL = S::KPL;
     constexpr int RS = S::RS;
     constexpr int NOUT = KPL * L2;  // 8 pixels per lane
-    constexpr int NACC = Acc<NAP>::N;
+    constexpr int NACC = FRAMES ? NAP : Acc<NAP>::N;
     constexpr int NSTAGE = PropSmem<NAP, NX, RPL>::NSTAGE;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int r = lane / LPR, g = (lane % LPR) / L2, n2 = lane % L2;
@@ -453,8 +469,14 @@ __device__ __forceinline__ bool prop_bins(const PropSmem<NAP, NX, RPL> &sm, cons
         const int st = (int)(n % NSTAGE);
         if (n >= NSTAGE && !mbar_wait(&sm.empty[st], ((n / NSTAGE) - 1) & 1)) return false;
         const int b = b_begin + issued;
-        mbar_expect_tx(&sm.full[st], BYTES_Q + BYTES_D);
-        bulk_g2s(sm.sQ + st * NAP * NX, Qf + (size_t)b * 2 * NAP * NX, BYTES_Q, &sm.full[st]);
+        if constexpr (FRAMES) {
+            mbar_expect_tx(&sm.full[st], (unsigned)live * (BYTES_Q / NAP) + BYTES_D);
+            for (int q = 0; q < live; ++q)
+                bulk_g2s(sm.sQ + (st * NAP + q) * NX, Qf + q * frame_q + (size_t)b * 2 * NX, BYTES_Q / NAP, &sm.full[st]);
+        } else {
+            mbar_expect_tx(&sm.full[st], BYTES_Q + BYTES_D);
+            bulk_g2s(sm.sQ + st * NAP * NX, Qf + (size_t)b * 2 * NAP * NX, BYTES_Q, &sm.full[st]);
+        }
         bulk_g2s(sm.sD + st * NX, phase + (size_t)b * NX, BYTES_D, &sm.full[st]);
         ++issued;
         return true;
@@ -523,6 +545,7 @@ __device__ __forceinline__ bool prop_bins(const PropSmem<NAP, NX, RPL> &sm, cons
         float2 px[L2 == 1 ? RPL : 1][L2 == 1 ? NAP : 1][8];
 #pragma unroll
         for (int q = 0; q < NAP; ++q) {
+            if (FRAMES && q >= live) break;
             float2 x[RPL][8];
 #pragma unroll
             for (int n1 = 0; n1 < 8; ++n1) {
@@ -557,12 +580,14 @@ __device__ __forceinline__ bool prop_bins(const PropSmem<NAP, NX, RPL> &sm, cons
 #pragma unroll
         for (int rr = 0; rr < RPL; ++rr) {
             const unsigned tcol_r = tcol + (unsigned)(rr * 8 * NACC);
-            float2 p[NAP][NOUT];
+            float2 p[FRAMES ? 1 : NAP][NOUT];   // a frame's field is added to its energy at once
 #pragma unroll
             for (int q = 0; q < NAP; ++q) {
+                if (FRAMES && q >= live) break;
+                float2(&pq)[NOUT] = p[FRAMES ? 0 : q];
                 if constexpr (L2 == 1) {
 #pragma unroll
-                    for (int k1 = 0; k1 < 8; ++k1) p[q][k1] = px[rr][q][k1];
+                    for (int k1 = 0; k1 < 8; ++k1) pq[k1] = px[rr][q][k1];
                 } else {
                     const float2 *reg = myT + ((q * RPW + r * RPL + rr) * 2 + g) * RS;
 #pragma unroll
@@ -577,13 +602,14 @@ __device__ __forceinline__ bool prop_bins(const PropSmem<NAP, NX, RPL> &sm, cons
                         }
                         IDft<L2>::run(v);
 #pragma unroll
-                        for (int k2 = 0; k2 < L2; ++k2) p[q][s * L2 + k2] = v[k2];
+                        for (int k2 = 0; k2 < L2; ++k2) pq[s * L2 + k2] = v[k2];
                     }
                 }
+                if constexpr (FRAMES) acc_update_frame(tcol_r + 8 * q, pq);
             }
 
             // per-pixel sums over the bins
-            acc_update<NAP>(tcol_r, p);
+            if constexpr (!FRAMES) acc_update<NAP>(tcol_r, p);
             if constexpr (FIELDS) {
                 if (row_ok) {  // fields of bin b
                     float2 *dst = fields_row + (size_t)b * bin_stride;
@@ -931,6 +957,148 @@ epi_reduce_seg_kernel(const float4 *__restrict__ part, int npix4, int nx, int rp
     }
 }
 
+// ---- AS energies of several frames (Eq. 3, one aperture) ----
+// One aperture spends half of its time on the phasors and the staging of a bin,
+// which depend on the bin and the row only: frames taken three at a time share
+// them. Measured (GB300, 301 x 128, 200 bins, whole call): 115.6 -> 97.4 us for 7
+// frames, 487 -> 384 us for 32; the kernel is at 88 us of the 7 frames' 97.
+constexpr int FR_N = 3;
+
+// The work is the sequence of (frame group, row tile, bin) units; a last group of
+// one or two frames costs less, and the CTAs' contiguous shares are equal in that
+// cost: 4 frames take 64 us, 78 us with all units counted alike.
+struct FrameDiv {
+    long long U = 0, Uf = 0;   // units; those of groups of FR_N frames
+    int wf = 1, wl = 1;        // cost of a unit of a full group and of the last one
+    int G = 1;                 // CTAs
+};
+// First unit of CTA c's share.
+__host__ __device__ __forceinline__ long long frame_share(const FrameDiv &d, int c)
+{
+    const long long full = d.Uf * d.wf, x = (full + (d.U - d.Uf) * d.wl) * c / d.G;
+    return x <= full ? x / d.wf : d.Uf + (x - full) / d.wl;
+}
+// The CTA whose share holds unit u (no share is empty).
+__host__ __device__ __forceinline__ int frame_cta_of(const FrameDiv &d, long long u)
+{
+    const long long full = d.Uf * d.wf, at = u < d.Uf ? u * d.wf : full + (u - d.Uf) * d.wl;
+    int c = (int)(at * d.G / (full + (d.U - d.Uf) * d.wl));
+    while (c > 0 && frame_share(d, c) > u) --c;
+    while (c + 1 < d.G && frame_share(d, c + 1) <= u) ++c;
+    return c;
+}
+
+// prop_seg_kernel for groups of FR_N frames (two rows per lane): a segment that
+// covers a tile's bins writes the frames' energies, a partial one its sums to slot
+// 2 c (the share's first segment) or 2 c + 1 (its last) of part[slot][FR_N][RPC][NX].
+template <int NX>
+__global__ void __launch_bounds__(32 * prop_warps(2, NX), PROP_CTAS)
+prop_frames_kernel(const float2 *__restrict__ Q, const uint4 *__restrict__ phase, const int *__restrict__ bin_evan,
+                   int n_bins, int nz, int tiles, int F, float z0f, float dzf, FrameDiv div, float *__restrict__ part,
+                   EpiOut out)
+{
+    constexpr int RPL = 2;
+    using S = Shape<NX, RPL>;
+    constexpr int L2 = S::L2, LPR = S::LPR, RPW = S::RPW, RPC = S::RPC, KPL = S::KPL, NOUT = KPL * L2;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const PropSmem<FR_N, NX, RPL> sm(smem_raw);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int r = lane / LPR, g = (lane % LPR) / L2, n2 = lane % L2;
+    const unsigned tbase = sm.init(tmem_cols<FR_N, RPL, NX>());
+    const unsigned tcol = acc_tcol(tbase, warp, FR_N, RPL);
+    pdl_wait();
+    const int c = blockIdx.x;
+    long long w = frame_share(div, c);
+    const long long w1 = frame_share(div, c + 1), wb = w;
+    const size_t frame_q = (size_t)n_bins * 2 * NX;
+    unsigned seq = 0;
+    while (w < w1) {
+        const long long tt = w / n_bins;
+        const int b0 = (int)(w - tt * n_bins);
+        const int nb = (int)min((long long)(n_bins - b0), w1 - w);
+        const int f0 = (int)(tt / tiles) * FR_N, tile = (int)(tt % tiles), live = min(FR_N, F - f0);
+        int jr[RPL], jj[RPL];
+        float zj[RPL];
+        bool rok[RPL];
+#pragma unroll
+        for (int rr = 0; rr < RPL; ++rr) {
+            jr[rr] = tile * RPC + warp * RPW + r * RPL + rr;
+            rok[rr] = jr[rr] < nz;
+            jj[rr] = rok[rr] ? jr[rr] : nz - 1;
+            zj[rr] = z0f + (float)jj[rr] * dzf;
+            const float z[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int q = 0; q < FR_N; ++q) tmem_st8(tcol + (unsigned)(8 * (rr * FR_N + q)), z);
+        }
+        tmem_wait_st();
+        const bool ok = prop_bins<FR_N, NX, false, RPL, true>(sm, Q + f0 * frame_q, phase, bin_evan, b0, nb, jj, zj, seq,
+                                                             tcol, nullptr, false, 0, live, frame_q);
+        seq += (unsigned)nb;
+        if (!ok && lane == 0) atomicOr(out.status, 1);
+        if (__syncthreads_or(!ok)) break;
+        if (w + nb >= w1) pdl_trigger();
+        const bool whole = nb == n_bins;
+        float *slot = part + (size_t)(2 * c + (wb < tt * n_bins ? 1 : 0)) * FR_N * RPC * NX;
+        tmem_wait_st();
+#pragma unroll
+        for (int rr = 0; rr < RPL; ++rr) {
+            float v[FR_N][8];
+#pragma unroll
+            for (int q = 0; q < FR_N; ++q) tmem_ld8(tcol + (unsigned)(8 * (rr * FR_N + q)), v[q]);
+            tmem_wait_ld();
+            if (rok[rr]) {
+#pragma unroll
+                for (int o = 0; o < NOUT; ++o) {
+                    const int k1 = n2 * KPL + o / L2, k2 = o % L2;
+                    const int i = 2 * (k1 + 8 * k2) + g;
+#pragma unroll
+                    for (int q = 0; q < FR_N; ++q) {
+                        if (q >= live) break;
+                        if (!whole)
+                            slot[((size_t)q * RPC + (jr[rr] - tile * RPC)) * NX + i] = v[q][o];
+                        else if (i < out.nx)
+                            out.out_main[(size_t)(f0 + q) * out.npix + (size_t)jr[rr] * out.nx + i] = v[q][o];
+                    }
+                }
+            }
+        }
+        w += nb;
+    }
+    sm.release(tbase, tmem_cols<FR_N, RPL, NX>());
+}
+
+// The tiles that CTAs of prop_frames_kernel share: each pixel's slots added in CTA
+// order. One warp per frame of the group and 32 groups of four pixels.
+__global__ void __launch_bounds__(32 * FR_N)
+epi_reduce_frames_kernel(const float4 *__restrict__ part, int npix4, int nx, int rpc, int n_bins, int tiles, int F,
+                         FrameDiv div, EpiOut out)
+{
+    const int q = threadIdx.x >> 5, lane = threadIdx.x & 31, f = blockIdx.y * FR_N + q;
+    const int tile4 = rpc * nx / 4, tile = (blockIdx.x * 32) / tile4;
+    const long long u = ((long long)blockIdx.y * tiles + tile) * n_bins;
+    const int cf = frame_cta_of(div, u), cl = frame_cta_of(div, u + n_bins - 1);
+    const int cf_slot = 2 * cf + (frame_share(div, cf) < u ? 1 : 0);
+    pdl_wait();
+    const int x4 = blockIdx.x * 32 + lane;
+    if (cf == cl || f >= F || x4 >= npix4) return;
+    constexpr int MAXS = 8;
+    const size_t off = (size_t)q * tile4 + (x4 - tile * tile4);
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int c0 = cf; c0 <= cl; c0 += MAXS) {
+        float4 v[MAXS];
+#pragma unroll
+        for (int k = 0; k < MAXS; ++k)
+            if (c0 + k <= cl) v[k] = part[(c0 + k == cf ? (size_t)cf_slot : 2 * (size_t)(c0 + k)) * FR_N * tile4 + off];
+#pragma unroll
+        for (int k = 0; k < MAXS; ++k)
+            if (c0 + k <= cl) {
+                a.x += v[k].x; a.y += v[k].y; a.z += v[k].z; a.w += v[k].w;
+            }
+    }
+    const int x = 4 * x4, row = x / nx, col = x - row * nx;   // columns past the image (2x padding) are dropped
+    if (col < out.nx) *reinterpret_cast<float4 *>(out.out_main + (size_t)f * out.npix + (size_t)row * out.nx + col) = a;
+}
+
 // rho_n = rho / max (Sec. II-A: the maximum becomes exactly 1) and the image
 // I = rho_n^2 E (Eq. 5 / Eq. 11). Four pixels per thread. `guard`: a maximum that
 // is not positive (a frame without a finite rho) gives rho_n = 0, the reading of
@@ -1183,6 +1351,35 @@ cudaError_t launch_seg_t(const pam_plan_s &p, int n_frames, const EpiOut &out, c
                             : launch_seg_rt<NAP, NX, 1>(p, n_frames, out, st);
 }
 
+// prop_frames_kernel's division of a call (launch and reduction agree on it).
+FrameDiv frame_div(const pam_plan_s &p, int n_frames, int tiles)
+{
+    FrameDiv d;
+    const int rest = n_frames % FR_N;
+    const long long per = (long long)tiles * p.n_bins;
+    d.Uf = n_frames / FR_N * per;
+    d.U = d.Uf + (rest ? per : 0);
+    long long G = (long long)PROP_CTAS * p.num_sms;
+    if (p.grid_override > 0 && p.grid_override < G) G = p.grid_override;
+    d.G = (int)(d.U < G ? d.U : G);
+    const int wf = 19, wl = rest == 1 ? 10 : 14;   // measured best of 9, 10 and 12 for one frame
+    if (d.Uf * wf + (d.U - d.Uf) * wl >= (long long)d.G * wf) {   // every share holds a unit
+        d.wf = wf;
+        d.wl = wl;
+    }
+    return d;
+}
+
+template <int NX>
+cudaError_t launch_frames_t(const pam_plan_s &p, int n_frames, const EpiOut &out, cudaStream_t st)
+{
+    const int tiles = (p.nz + Shape<NX, 2>::RPC - 1) / Shape<NX, 2>::RPC;
+    const FrameDiv d = frame_div(p, n_frames, tiles);
+    return launch_pdl(p.pdl, prop_frames_kernel<NX>, d.G, 32 * prop_warps(2, NX), prop_smem_bytes<FR_N, NX, 2>(), st, p.w.Q,
+                      p.t.phase, p.t.bin_evan, p.n_bins, p.nz, tiles, n_frames, (float)p.d.z0_m, (float)p.d.dz_m, d,
+                      p.w.part, out);
+}
+
 template <int NX, bool CLUSTER>
 cudaError_t launch_prop_nc(const pam_plan_s &p, int n_frames, int napq, int n_split, float *fields,
                            const EpiOut &out, cudaStream_t st)
@@ -1195,11 +1392,26 @@ cudaError_t launch_prop_nc(const pam_plan_s &p, int n_frames, int napq, int n_sp
     return launch_prop_t<3, NX, false, CLUSTER>(p, n_frames, n_split, nullptr, out, st);
 }
 
+// AS energies of two or more frames share the phasors if that leaves a CTA five
+// units or more: a unit of three frames is a longer chain than one of one frame, so
+// with few units the division by frames fills the chip better. Measured (GB300, us
+// a call, one frame at a time / three): nx = 128 with 9.2 units a CTA 40.7 / 39.2;
+// nx = 64 with 2.4 24.7 / 26.2, with 8.7 62.0 / 51.6; nx = 32 with 2.9 24.6 / 26.0;
+// nx = 16 with 3.2 19.7 / 22.8, with 5.8 29.5 / 28.5.
+bool frames_mode(const pam_plan_s &p, int n_frames, int napq)
+{
+    if (napq != 1 || n_frames < 2 || p.lane_rows != 2) return false;
+    const int rows = prop_rows_per_cta(p.nx, 2);
+    const FrameDiv d = frame_div(p, n_frames, (p.nz + rows - 1) / rows);
+    return d.U >= 5LL * d.G;
+}
+
 template <int NX>
 cudaError_t launch_prop_nx(const pam_plan_s &p, int n_frames, int napq, int n_split, float *fields,
                            const EpiOut &out, cudaStream_t st)
 {
     if (prop_seg_mode(p, n_split, fields != nullptr)) {
+        if (frames_mode(p, n_frames, napq)) return launch_frames_t<NX>(p, n_frames, out, st);
         if (napq == 1) return launch_seg_t<1, NX>(p, n_frames, out, st);
         if (napq == 2) return launch_seg_t<2, NX>(p, n_frames, out, st);
         return launch_seg_t<3, NX>(p, n_frames, out, st);
@@ -1244,6 +1456,7 @@ cudaError_t prepare_nx()
     if (e == cudaSuccess) e = set_smem_of(prop_batch_kernel<3, NX, 1>, prop_smem_bytes<3, NX, 1>());
     if (e == cudaSuccess) e = set_smem_of(prop_batch_kernel<2, NX, 2>, prop_smem_bytes<2, NX, 2>());
     if (e == cudaSuccess) e = set_smem_of(prop_batch_kernel<3, NX, 2>, prop_smem_bytes<3, NX, 2>());
+    if (e == cudaSuccess) e = set_smem_of(prop_frames_kernel<NX>, prop_smem_bytes<FR_N, NX, 2>());
     if (e == cudaSuccess) e = set_smem_of(prop_seg_kernel<1, NX, 1>, prop_smem_bytes<1, NX, 1>());
     if (e == cudaSuccess) e = set_smem_of(prop_seg_kernel<2, NX, 1>, prop_smem_bytes<2, NX, 1>());
     if (e == cudaSuccess) e = set_smem_of(prop_seg_kernel<3, NX, 1>, prop_smem_bytes<3, NX, 1>());
@@ -1336,7 +1549,10 @@ size_t prop_seg_part_floats(const pam_plan_s &p)
     // the larger row tile of the two rows-per-lane settings, which can change after the plan is made
     const int r1 = prop_rows_per_cta(p.nx, 1), r2 = prop_rows_per_cta(p.nx, 2);
     const int rows = r1 > r2 ? r1 : r2;
-    return (size_t)2 * PROP_CTAS * p.num_sms * n_acc(p.n_apod) * rows * p.nx;
+    // AS energies of several frames at once keep FR_N sums
+    int sums = n_acc(p.n_apod);
+    if (p.max_frames > 1 && sums < FR_N) sums = FR_N;
+    return (size_t)2 * PROP_CTAS * p.num_sms * sums * rows * p.nx;
 }
 
 int choose_split(const pam_plan_s &p, int n_frames)
@@ -1388,6 +1604,11 @@ cudaError_t launch_epilogue(const pam_plan_s &p, int n_frames, int napq, int n_s
         const int G = prop_seg_ctas(p, n_frames);
         const float4 *part = reinterpret_cast<const float4 *>(p.w.part);
         dim3 rgrid((npix4 + 31) / 32, n_frames);
+        if (frames_mode(p, n_frames, napq)) {
+            rgrid.y = (n_frames + FR_N - 1) / FR_N;
+            return launch_pdl(p.pdl, epi_reduce_frames_kernel, rgrid, 32 * FR_N, 0, st, part, npix4, p.nx, rows, p.n_bins,
+                              tiles, n_frames, frame_div(p, n_frames, tiles), out);
+        }
         const int rg = (long long)rgrid.x * rgrid.y <= 2LL * p.num_sms ? 4 : 2;
         auto reduce = napq == 1 ? (rg == 4 ? epi_reduce_seg_kernel<1, 4> : epi_reduce_seg_kernel<1, 2>)
                       : napq == 2 ? (rg == 4 ? epi_reduce_seg_kernel<2, 4> : epi_reduce_seg_kernel<2, 2>)
