@@ -56,7 +56,9 @@ constexpr int DFT_MAX_NT = 16384;
 // its own and then added to the total, so the rounding error grows like
 // 64 + nt/64 ulp rather than nt ulp.
 // Measured (GB300, 64 frames of 128 channels, 1024-8192 samples, 300 bins):
-// 1.24 ms against 2.27 ms (FMA pipe 65% busy, two warps per scheduler).
+// 1.24 ms against 2.27 ms (FMA pipe 65% busy, two warps per scheduler). More warps
+// do not help: with the totals in tensor memory three CTAs per SM take 1.24 ms and
+// four (128 registers) 1.40 ms.
 constexpr int XROW = DFT_T + 4;     // floats per staged channel row
 constexpr int WROW = DFT_T + 2;     // float2 per staged twiddle row (16-byte rows)
 
