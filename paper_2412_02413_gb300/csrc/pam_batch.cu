@@ -358,7 +358,7 @@ pam_status enqueue(pam_batch_s *b, const float *rf, float *image, float *rho_n, 
                                                  ((size_t)pam::n_acc(b->napq) * pam::prop_rows_per_cta(b->nx, b->rpl) * b->nx));
     // persistent CTAs for each bin chunk of the items, at most one per SM altogether
     const int units = pam::item_units(k.n_items, k.sms, k.cap), chunks = units / k.n_items;
-    k.grid = std::min(units, b->grid_override > 0 ? b->grid_override * chunks
+    k.grid = std::min(units, b->grid_override > 0 ? std::min(b->grid_override, k.n_items) * chunks
                                                   : pam::prop_ctas_per_sm() * p.num_sms);
     e = pam::launch_prop_batch(b->nx, b->napq, k, out, st, b->rpl);
     if (e != cudaSuccess) return pam::cuda_fail(e, "propagate/correlate launch");

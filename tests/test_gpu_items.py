@@ -93,3 +93,19 @@ def test_captured_call_equals_the_eager_one():
     assert torch.equal(ge, e)
     for k, v in out.items():
         assert torch.equal(got[k], v), k
+
+
+@pytest.mark.parametrize("use_graph", [False, True])
+def test_any_positive_grid_is_taken(use_graph):
+    """A grid above the item count stands for the items' whole work, up to the
+    largest number the interface takes."""
+    b = _pam().Batch(n_elem=64, pitch=PITCH, fs=FS, c=C, frames=[(1024, 40)], z0=Z0, dz=DZ, n_bins=300, f_lo=1e6,
+                     f_hi=8e6, n_apod=3, pattern_m=2)
+    rf = b.pack_rf([synth.random_rf(64, 1024, seed=890)])
+    img, rn = (t.clone() for t in b.as_tax(rf))
+    for ctas in (2, 153, 2 ** 31 // 48, 2 ** 31 - 1):
+        b.configure(use_graph=use_graph, persistent_ctas=ctas)
+        img1, rn1 = b.as_tax(rf)
+        torch.cuda.synchronize()
+        assert torch.equal(img1, img) and torch.equal(rn1, rn), ctas
+    b.sync()
