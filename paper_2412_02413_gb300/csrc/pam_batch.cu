@@ -251,6 +251,7 @@ struct pam_batch_s {
     pam_plan_s *base = nullptr;     // geometry, apodization, workspace for F frames of n_bins bins
     int F = 0, n_bins = 0, ne = 0, nx = 0, napq = 0, max_npix = 0, cpl = 4;
     int grid = 0, grid_override = 0, n_items = 0;
+    int split = 1;                   // bin chunks per item
     int rpl = 1;                     // depth rows per lane of the fused kernel (2 for nx >= 64)
     std::vector<int> nt, nz, nbf, bins_h;   // per frame: samples, rows, bin count; bins [F][n_bins]
     std::vector<size_t> rf_off, px_off;
@@ -275,10 +276,6 @@ struct pam_batch_s {
 };
 
 namespace {
-
-// Work units (items times bin chunks) up to which items are split: 150 MB of
-// partial sums at nx = 128, within the workspace of the batches that need it.
-constexpr size_t kMaxUnits = 1024;
 
 void batch_free(pam_batch_s *b)
 {
@@ -352,19 +349,16 @@ pam_status enqueue(pam_batch_s *b, const float *rf, float *image, float *rho_n, 
     k.items = b->items;
     k.n_items = b->n_items;
     k.counter = b->counter;
-    k.sms = p.num_sms;
+    k.split = b->split;
     k.part = p.w.part;
-    k.cap = (int)std::min<size_t>(kMaxUnits, p.w.part_floats /
-                                                 ((size_t)pam::n_acc(b->napq) * pam::prop_rows_per_cta(b->nx, b->rpl) * b->nx));
     // persistent CTAs for each bin chunk of the items, at most one per SM altogether
-    const int units = pam::item_units(k.n_items, k.sms, k.cap), chunks = units / k.n_items;
-    k.grid = std::min(units, b->grid_override > 0 ? std::min(b->grid_override, k.n_items) * chunks
-                                                  : pam::prop_ctas_per_sm() * p.num_sms);
+    k.grid = std::min(k.n_items * k.split, b->grid_override > 0 ? std::min(b->grid_override, k.n_items) * k.split
+                                                                : pam::prop_ctas_per_sm() * p.num_sms);
     e = pam::launch_prop_batch(b->nx, b->napq, k, out, st, b->rpl);
     if (e != cudaSuccess) return pam::cuda_fail(e, "propagate/correlate launch");
     e = pam::launch_normalize_batch(b->F, b->max_npix, b->frames, out, st);
     if (e != cudaSuccess) return pam::cuda_fail(e, "normalise launch");
-    b->n_kernels = 3 + pam::prop_batch_kernels(k);
+    b->n_kernels = k.split > 1 ? 5 : 4;
     b->kernels += b->n_kernels;
     return PAM_OK;
 }
@@ -456,6 +450,8 @@ pam_status pam_batch_create(const pam_plan_desc *common, const pam_frame_desc *f
         for (int t = 0; t * rpc < b->nz[f]; ++t) items.push_back(make_int2(f, t));
     b->n_items = (int)items.size();
     b->grid = std::min(b->n_items, pam::prop_ctas_per_sm() * p.num_sms);
+    b->split = pam::item_split(b->nx, b->napq, b->rpl, b->n_items, *std::max_element(b->nbf.begin(), b->nbf.end()),
+                               p.num_sms, p.w.part_floats);
     const size_t FB = (size_t)n_frames * b->n_bins;
     cudaError_t e = cudaSuccess;
     if (e == cudaSuccess) e = dalloc(&b->bins, FB);

@@ -66,11 +66,10 @@ struct ItemWork {
     const BatchFrame *frames = nullptr;
     const int2 *items = nullptr;         // (frame, row tile of prop_rows_per_cta(nx, rpl) rows)
     int n_items = 0;
-    const int *n_items_dev = nullptr;    // optional: a device int that caps n_items when the kernel starts
+    const int *n_items_dev = nullptr;    // optional (split 1): a device int that caps n_items when the kernel starts
     int *counter = nullptr;              // work-queue head, zero before the launch
-    int sms = 0;                         // SMs the bins of few items are split over
-    float *part = nullptr;               // `cap` slots of n_acc x rows x nx floats for the split items' sums
-    int cap = 0;                         // (fewer than 2: items are not split)
+    int split = 1;                       // bin chunks per item (item_split)
+    float *part = nullptr;               // split > 1: n_items * split slots of n_acc x rows x nx floats for their sums
 };
 
 struct Workspace {
@@ -202,8 +201,8 @@ size_t prop_seg_part_floats(const pam_plan_s &p);
 // normalisation.
 // rpl: depth rows per lane; the items' row tiles are prop_rows_per_cta(nx, rpl) rows.
 cudaError_t launch_prop_batch(int nx, int napq, const ItemWork &k, const EpiOut &out, cudaStream_t st, int rpl);
-int prop_batch_kernels(const ItemWork &k);               // kernels it launches
-int item_units(int n_items, int sms, int cap);           // items times their bin chunks
+// Bin chunks per item: n_bins bins of the longest frame, `floats` of Workspace::part.
+int item_split(int nx, int napq, int rpl, int n_items, int n_bins, int sms, size_t floats);
 // Full-aperture energy split by bins: the fused kernel (one aperture, whatever
 // Q holds) over n_bands contiguous chunks of Omega, chunk b = bins
 // [floor(n_bins b / n_bands), floor(n_bins (b+1) / n_bands)), each chunk's

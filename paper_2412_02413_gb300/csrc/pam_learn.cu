@@ -882,12 +882,11 @@ cudaError_t run_items(pam_learn_s *l, const int2 *items, int n_items, const int 
     k.n_items = n_items;
     k.n_items_dev = n_items_dev;
     k.counter = head;
-    k.sms = l->n_sms;
     k.part = p.w.part;
-    if (spread) k.cap = (int)std::min<size_t>(1024, p.w.part_floats / ((size_t)6 * pam::prop_rows_per_cta(l->W, rpl) * l->W));
+    if (spread) k.split = pam::item_split(l->W, 3, rpl, n_items, p.n_bins, l->n_sms, p.w.part_floats);
     const int ctas = pam::prop_ctas_per_sm() * l->n_sms;
-    k.grid = n_items_dev ? ctas : std::min(ctas, pam::item_units(n_items, k.sms, k.cap));
-    l->kernels += pam::prop_batch_kernels(k);
+    k.grid = n_items_dev ? ctas : std::min(ctas, n_items * k.split);
+    l->kernels += k.split > 1 ? 2 : 1;
     return pam::launch_prop_batch(l->W, 3, k, out, st, rpl);
 }
 

@@ -23,6 +23,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "pam_internal.h"
 #include "pam_ptx.h"
 
@@ -1121,31 +1123,6 @@ epi_normalize_kernel(const float4 *__restrict__ rho_tmp, const float4 *__restric
     if (rho_n) rho_n[o] = rn;
 }
 
-// Bin chunks per work item of prop_batch_kernel: one where the items fill the
-// SMs, more where a few items (or a last wave of few) would leave most of them
-// idle. The split that minimises waves x (chunk time + the cost of a partial: its
-// sums go to memory and back, about 10 us against 1 ms for an item's 300 bins at
-// nx = 128), at most kMaxItemSplit and what `cap` slots of partial sums hold.
-// It depends on the items and the device alone, not on the grid, so that a
-// launch's grouping of the sums, and with it every bit, does not depend on the
-// grid. Measured (GB300): the gate tiles of 32 frames (32 items of 32 rows x 300
-// bins) 175 us and 26 us for the sums, against 705 us unsplit.
-constexpr int kMaxItemSplit = 48;
-__host__ __device__ __forceinline__ int item_split(int n_items, int sms, int cap)
-{
-    int best = 1, cost = 0x7fffffff;
-    for (int s = 1; s <= kMaxItemSplit; ++s) {
-        if (s > 1 && (long long)n_items * s > cap) break;
-        const int waves = (int)(((long long)n_items * s + sms - 1) / sms);
-        const long long c = (long long)waves * (10000 / s + (s > 1 ? 100 : 0));
-        if (c < cost) {
-            cost = (int)c;
-            best = s;
-        }
-    }
-    return best;
-}
-
 // Persistent form for a batch of frames with their own bins and depth grids
 // (uneven sample counts and depth ranges). Work units are (frame, row tile)
 // items times the bin chunks of item_split, taken from a global counter. With
@@ -1156,11 +1133,10 @@ __host__ __device__ __forceinline__ int item_split(int n_items, int sms, int cap
 template <int NAP, int NX, int RPL>
 __global__ void __launch_bounds__(32 * prop_warps(RPL, NX), PROP_CTAS)
 prop_batch_kernel(const BatchFrame *__restrict__ frames, const int2 *__restrict__ items, int n_items,
-                  const int *__restrict__ n_items_dev, int *__restrict__ counter, int sms, int cap,
+                  const int *__restrict__ n_items_dev, int *__restrict__ counter, int split,
                   float *__restrict__ part, EpiOut out)
 {
     if (n_items_dev) n_items = min(n_items, *n_items_dev);
-    const int split = item_split(n_items, sms, cap);
     using S = Shape<NX, RPL>;
     constexpr int L2 = S::L2, LPR = S::LPR, RPW = S::RPW, RPC = S::RPC, KPL = S::KPL;
     constexpr int NACC = Acc<NAP>::N;
@@ -1238,54 +1214,48 @@ prop_batch_kernel(const BatchFrame *__restrict__ frames, const int2 *__restrict_
 template <int NAP>
 __global__ void __launch_bounds__(32 * Acc<NAP>::N)
 epi_reduce_items_kernel(const float4 *__restrict__ part, const BatchFrame *__restrict__ frames,
-                        const int2 *__restrict__ items, int n_items, const int *__restrict__ n_items_dev, int sms,
-                        int cap, int nx, int rpc, EpiOut out)
+                        const int2 *__restrict__ items, int split, int nx, int rpc, EpiOut out)
 {
     constexpr int NACC = Acc<NAP>::N;
-    if (n_items_dev) n_items = min(n_items, *n_items_dev);
-    const int split = item_split(n_items, sms, cap);
-    if (split == 1) return;
     __shared__ float4 sA[NACC][32];
     __shared__ float wmax[NACC];
     const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tile4 = rpc * nx / 4;
     const int x4 = blockIdx.x * 32 + lane, x = 4 * x4, row = x / nx, col = x - row * nx;
-    for (int it = blockIdx.y; it < n_items; it += gridDim.y) {
-        const int2 w = items[it];
-        const BatchFrame fr = frames[w.x];
-        const int j = w.y * rpc + row;
-        const bool live = x4 < tile4 && j < fr.nz;
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (live) {
-            // a chunk's loads are issued 8 at a time ahead of the sums
-            const float4 *src = part + ((size_t)it * split * NACC + c) * tile4 + x4;
-            for (int s0 = 0; s0 < split; s0 += 8) {
-                float4 v[8];
+    const int it = blockIdx.y;
+    const int2 w = items[it];
+    const BatchFrame fr = frames[w.x];
+    const int j = w.y * rpc + row;
+    const bool live = x4 < tile4 && j < fr.nz;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (live) {
+        // a chunk's loads are issued 8 at a time ahead of the sums
+        const float4 *src = part + ((size_t)it * split * NACC + c) * tile4 + x4;
+        for (int s0 = 0; s0 < split; s0 += 8) {
+            float4 v[8];
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    if (s0 + k < split) v[k] = src[(size_t)(s0 + k) * NACC * tile4];
+            for (int k = 0; k < 8; ++k)
+                if (s0 + k < split) v[k] = src[(size_t)(s0 + k) * NACC * tile4];
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    if (s0 + k < split) {
-                        a.x += v[k].x; a.y += v[k].y; a.z += v[k].z; a.w += v[k].w;
-                    }
-            }
+            for (int k = 0; k < 8; ++k)
+                if (s0 + k < split) {
+                    a.x += v[k].x; a.y += v[k].y; a.z += v[k].z; a.w += v[k].w;
+                }
         }
-        sA[c][lane] = a;
-        __syncthreads();
-        float rmax = 0.0f;
-        if (c == 0 && live) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                float acc[NACC];
-#pragma unroll
-                for (int k = 0; k < NACC; ++k) acc[k] = reinterpret_cast<const float *>(&sA[k][lane])[i];
-                rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc, out, fr.out_off, j, col + i));
-            }
-        }
-        block_max_to(rmax, out.fmax + w.x, wmax, 32 * NACC);
-        __syncthreads();
     }
+    sA[c][lane] = a;
+    __syncthreads();
+    float rmax = 0.0f;
+    if (c == 0 && live) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float acc[NACC];
+#pragma unroll
+            for (int k = 0; k < NACC; ++k) acc[k] = reinterpret_cast<const float *>(&sA[k][lane])[i];
+            rmax = fmaxf(rmax, pixel_epilogue<NAP>(acc, out, fr.out_off, j, col + i));
+        }
+    }
+    block_max_to(rmax, out.fmax + w.x, wmax, 32 * NACC);
 }
 
 // Per-frame rho_n and image for a batch packed by per-frame pixel offsets.
@@ -1471,13 +1441,12 @@ cudaError_t launch_batch_t(const ItemWork &k, const EpiOut &out, cudaStream_t st
 {
     static_assert(prop_smem_bytes<NAP, NX, RPL>() + 1024 <= 232448, "shared memory of the fused kernel");
     prop_batch_kernel<NAP, NX, RPL><<<k.grid, 32 * prop_warps(RPL, NX), prop_smem_bytes<NAP, NX, RPL>(), st>>>(
-        k.frames, k.items, k.n_items, k.n_items_dev, k.counter, k.sms, k.cap, k.part, out);
+        k.frames, k.items, k.n_items, k.n_items_dev, k.counter, k.split, k.part, out);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || prop_batch_kernels(k) == 1) return e;
+    if (e != cudaSuccess || k.split == 1) return e;
     constexpr int RPC = Shape<NX, RPL>::RPC;
-    const int most = k.cap / 2 < k.n_items ? k.cap / 2 : k.n_items;   // items that can be split
-    epi_reduce_items_kernel<NAP><<<dim3((RPC * NX / 4 + 31) / 32, most), 32 * Acc<NAP>::N, 0, st>>>(
-        reinterpret_cast<const float4 *>(k.part), k.frames, k.items, k.n_items, k.n_items_dev, k.sms, k.cap, NX, RPC, out);
+    epi_reduce_items_kernel<NAP><<<dim3((RPC * NX / 4 + 31) / 32, k.n_items), 32 * Acc<NAP>::N, 0, st>>>(
+        reinterpret_cast<const float4 *>(k.part), k.frames, k.items, k.split, NX, RPC, out);
     return cudaGetLastError();
 }
 
@@ -1633,12 +1602,40 @@ cudaError_t launch_epilogue(const pam_plan_s &p, int n_frames, int napq, int n_s
                       st, v4(out.rho_tmp), v4(out.e_tmp), out.fmax, out4, out.nx != p.nx, v4(out.out_main), v4(out.rho_n));
 }
 
-int item_units(int n_items, int sms, int cap) { return n_items * item_split(n_items, sms, cap); }
-
-int prop_batch_kernels(const ItemWork &k)
+// Bin chunks per work item of prop_batch_kernel: one where the items fill the
+// SMs, more where a few items (or a last wave of few) would leave most of them
+// idle. The split with the least estimated time
+//   waves x bins per chunk x time of a bin + (with a second kernel) 6 us + 60 ns a unit,
+// where a bin takes 0.50 ns a pixel of the row tile (DAX: 0.36) and a unit's sums go
+// to memory and back. At most a chunk per bin, kMaxItemSplit, kMaxItemUnits and what
+// `floats` of partial sums hold. It depends on the batch and the device alone, not on
+// the grid, so that a launch's grouping of the sums, and with it every bit, does not
+// depend on the grid.
+// Measured (GB300, whole calls, us, unsplit / this split): nx = 128, 9 items 1058 / 141
+// with 300 bins, 77 / 51 with 10; nx = 32, 4 items 128 / 48 with 40. Against the best of
+// splits 1 to 48 over widths 16 to 128, 1 to 180 items and 3 to 300 bins it is 1.3 %
+// slower on average and never more than the timer's step slower than unsplit, where a
+// rule without bins and width (48 chunks for one item) took 130 for 107 us (nx = 64,
+// 100 items of 5 bins). The gate tiles of 32 frames (32 items of 32 rows x 300 bins at
+// nx = 128) take 175 us and 26 us for the sums, against 705 us unsplit.
+constexpr int kMaxItemSplit = 48, kMaxItemUnits = 1024;
+int item_split(int nx, int napq, int rpl, int n_items, int n_bins, int sms, size_t floats)
 {
-    // with the count on the device the split is known there only
-    return k.cap >= 2 && (k.n_items_dev || item_split(k.n_items, k.sms, k.cap) > 1) ? 2 : 1;
+    const int tile = prop_rows_per_cta(nx, rpl) * nx;
+    const long long slots = std::min<long long>(kMaxItemUnits, (long long)(floats / ((size_t)n_acc(napq) * tile)));
+    const long long t_bin = (long long)tile * (napq == 3 ? 50 : 36) / 100;   // ns
+    int best = 1;
+    long long least = 0;
+    for (int s = 1; s <= kMaxItemSplit && s <= n_bins; ++s) {
+        const long long units = (long long)n_items * s;
+        if (s > 1 && units > slots) break;
+        const long long ns = (units + sms - 1) / sms * ((n_bins + s - 1) / s) * t_bin + (s > 1 ? 6000 + 60 * units : 0);
+        if (s == 1 || ns < least) {
+            least = ns;
+            best = s;
+        }
+    }
+    return best;
 }
 
 cudaError_t launch_prop_batch(int nx, int napq, const ItemWork &k, const EpiOut &out, cudaStream_t st, int rpl)

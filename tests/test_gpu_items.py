@@ -109,3 +109,21 @@ def test_any_positive_grid_is_taken(use_graph):
         torch.cuda.synchronize()
         assert torch.equal(img1, img) and torch.equal(rn1, rn), ctas
     b.sync()
+
+
+@pytest.mark.parametrize("ne,frames,n_bins,kernels", [
+    (64, [(1024, 400)] * 20, 3, 4),             # 100 items of 3 bins: dividing them costs more than it saves
+    (16, [(64, 40)], 1, 4),                     # one bin cannot be divided
+    (128, [(1024, 400)], 300, 5),               # 9 items of 300 bins
+])
+def test_items_are_divided_where_their_bins_pay_for_it(ne, frames, n_bins, kernels):
+    b = _pam().Batch(n_elem=ne, pitch=PITCH, fs=FS, c=C, frames=frames, z0=Z0, dz=0.1e-3, n_bins=n_bins, f_lo=1e6,
+                     f_hi=8e6, n_apod=3, pattern_m=2)
+    rf = b.pack_rf([synth.random_rf(ne, nt, seed=895) for nt, _ in frames])
+    img, rn = (t.clone() for t in b.as_tax(rf))
+    assert b.info()[2] == kernels
+    b.configure(use_graph=False, persistent_ctas=1)
+    img1, rn1 = b.as_tax(rf)
+    torch.cuda.synchronize()
+    b.sync()
+    assert torch.equal(img1, img) and torch.equal(rn1, rn)
