@@ -372,13 +372,15 @@ pam_status pam_batch_sync(pam_batch_t b, void *stream);
 
 /* Tuning knobs. use_graph 0 launches the kernels directly (no graph);
  * persistent_ctas > 0 sets the grid of the persistent kernel (0: one per SM,
- * the most that fit; at most one per work item; for each chunk of the bins where
- * few work items have theirs divided). Results do not depend on it. */
+ * the most that fit; at most one per work item). Where few work items have their
+ * bins divided into chunks, it is the CTAs for each chunk, and 0 launches one per
+ * SM at most altogether. Results do not depend on it. */
 pam_status pam_batch_configure(pam_batch_t b, int use_graph, int persistent_ctas);
 
-/* Work items (frame, row tile), the persistent grid in use, and the libpam
- * kernels launched so far (a graph launch counts its 4 or 5 kernels). Any output
- * pointer may be NULL. */
+/* Work items (frame, row tile), the persistent grid in use in the units of
+ * pam_batch_configure (per chunk where the items' bins are divided: the launch has
+ * a multiple of it), and the libpam kernels launched so far (a graph launch counts
+ * its 4 kernels, 5 where the bins are divided). Any output pointer may be NULL. */
 pam_status pam_batch_info(pam_batch_t b, int *n_items, int *persistent_ctas, long long *kernel_launches);
 
 /* Frees the batch (NULL-safe). Waits for the device first. */

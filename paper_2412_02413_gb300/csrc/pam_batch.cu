@@ -325,6 +325,13 @@ pam_status frame_bins(const pam_plan_desc *c, const pam_frame_desc &fd, int n_bi
     return PAM_OK;
 }
 
+// Persistent CTAs for each chunk of the items' bins (one chunk unless few items
+// have theirs divided): the configured number, or one per SM, at most one per item.
+int ctas_per_chunk(const pam_batch_s *b)
+{
+    return b->grid_override > 0 ? std::min(b->grid_override, b->n_items) : b->grid;
+}
+
 pam_status enqueue(pam_batch_s *b, const float *rf, float *image, float *rho_n, cudaStream_t st)
 {
     pam_plan_s &p = *b->base;
@@ -351,9 +358,8 @@ pam_status enqueue(pam_batch_s *b, const float *rf, float *image, float *rho_n, 
     k.counter = b->counter;
     k.split = b->split;
     k.part = p.w.part;
-    // persistent CTAs for each bin chunk of the items, at most one per SM altogether
-    k.grid = std::min(k.n_items * k.split, b->grid_override > 0 ? std::min(b->grid_override, k.n_items) * k.split
-                                                                : pam::prop_ctas_per_sm() * p.num_sms);
+    k.grid = ctas_per_chunk(b) * k.split;
+    if (b->grid_override == 0) k.grid = std::min(k.grid, pam::prop_ctas_per_sm() * p.num_sms);
     e = pam::launch_prop_batch(b->nx, b->napq, k, out, st, b->rpl);
     if (e != cudaSuccess) return pam::cuda_fail(e, "propagate/correlate launch");
     e = pam::launch_normalize_batch(b->F, b->max_npix, b->frames, out, st);
@@ -603,7 +609,7 @@ pam_status pam_batch_info(pam_batch_t b, int *n_items, int *persistent_ctas, lon
 {
     if (!b) return pam::fail(PAM_ERR_INVALID_ARG, "batch is NULL");
     if (n_items) *n_items = b->n_items;
-    if (persistent_ctas) *persistent_ctas = b->grid_override > 0 ? std::min(b->grid_override, b->n_items) : b->grid;
+    if (persistent_ctas) *persistent_ctas = ctas_per_chunk(b);
     if (kernel_launches) *kernel_launches = b->kernels;
     return PAM_OK;
 }

@@ -498,7 +498,7 @@ class Batch:
         _check(load().pam_batch_configure(self._h, int(bool(use_graph)), int(persistent_ctas)))
 
     def info(self):
-        """(work items, persistent grid, libpam kernel launches so far)."""
+        """(work items, persistent grid as ``configure`` takes it, libpam kernel launches so far)."""
         n, g, k = ctypes.c_int(), ctypes.c_int(), ctypes.c_longlong()
         _check(load().pam_batch_info(self._h, ctypes.byref(n), ctypes.byref(g), ctypes.byref(k)))
         return n.value, g.value, k.value

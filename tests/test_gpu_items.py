@@ -108,6 +108,7 @@ def test_any_positive_grid_is_taken(use_graph):
         img1, rn1 = b.as_tax(rf)
         torch.cuda.synchronize()
         assert torch.equal(img1, img) and torch.equal(rn1, rn), ctas
+        assert b.info()[:2] == (1, 1)        # the grid as configure takes it: one CTA for each chunk of the one item
     b.sync()
 
 
