@@ -252,7 +252,7 @@ constexpr int TFFT_THREADS = 256;
 
 template <int MAXR>
 __global__ void __launch_bounds__(TFFT_THREADS)
-time_fft_kernel(const float *__restrict__ rf, int ne, int nt, int log2nt, const float2 *__restrict__ tw,
+time_fft_kernel(const float *rf, int ne, int nt, int log2nt, const float2 *__restrict__ tw,
                 const int *__restrict__ bins, int n_bins, float2 *__restrict__ S, int nev, int cstep,
                 unsigned *__restrict__ fmax)
 {
@@ -310,7 +310,7 @@ time_fft_kernel(const float *__restrict__ rf, int ne, int nt, int log2nt, const 
 constexpr int LAT_THREADS = 128;
 
 __global__ void __launch_bounds__(LAT_THREADS)
-lateral_kernel(const float2 *__restrict__ S, int ne, int nx, int log2nx, int n_bins, int napq,
+lateral_kernel(const float2 *S, int ne, int nx, int log2nx, int n_bins, int napq,
                const float *__restrict__ apod, const float2 *__restrict__ twx, const float *__restrict__ live,
                size_t live_fs, float2 *__restrict__ Q)
 {

@@ -759,7 +759,7 @@ __host__ __device__ __forceinline__ long long seg_slot(int c, long long tt, long
 // ring carries over from segment to segment.
 template <int NAP, int NX, int RPL>
 __global__ void __launch_bounds__(32 * prop_warps(RPL, NX), PROP_CTAS)
-prop_seg_kernel(const float2 *__restrict__ Q, const uint4 *__restrict__ phase, const int *__restrict__ bin_evan,
+prop_seg_kernel(const float2 *Q, const uint4 *__restrict__ phase, const int *__restrict__ bin_evan,
                 int n_bins, int nz, int tiles, float z0f, float dzf, long long W, float *__restrict__ part,
                 EpiOut out)
 {
@@ -892,7 +892,7 @@ epi_reduce_kernel(const float4 *__restrict__ part, int n_split, int npix4, int n
 // with 4, 7.8 with one, which took 10 us while one warp of six did the pixel math).
 template <int NAP, int RED_G>
 __global__ void __launch_bounds__(32 * RED_G * Acc<NAP>::N, NAP == 3 ? 8 / RED_G : 4)
-epi_reduce_seg_kernel(const float4 *__restrict__ part, int npix4, int nx, int rpc, int n_bins, int tiles, long long W,
+epi_reduce_seg_kernel(const float4 *part, int npix4, int nx, int rpc, int n_bins, int tiles, long long W,
                       int G, EpiOut out)
 {
     constexpr int NACC = Acc<NAP>::N;
@@ -995,7 +995,7 @@ __host__ __device__ __forceinline__ int frame_cta_of(const FrameDiv &d, long lon
 // 2 c (the share's first segment) or 2 c + 1 (its last) of part[slot][FR_N][RPC][NX].
 template <int NX>
 __global__ void __launch_bounds__(32 * prop_warps(2, NX), PROP_CTAS)
-prop_frames_kernel(const float2 *__restrict__ Q, const uint4 *__restrict__ phase, const int *__restrict__ bin_evan,
+prop_frames_kernel(const float2 *Q, const uint4 *__restrict__ phase, const int *__restrict__ bin_evan,
                    int n_bins, int nz, int tiles, int F, float z0f, float dzf, FrameDiv div, float *__restrict__ part,
                    EpiOut out)
 {
@@ -1072,7 +1072,7 @@ prop_frames_kernel(const float2 *__restrict__ Q, const uint4 *__restrict__ phase
 // The tiles that CTAs of prop_frames_kernel share: each pixel's slots added in CTA
 // order. One warp per frame of the group and 32 groups of four pixels.
 __global__ void __launch_bounds__(32 * FR_N)
-epi_reduce_frames_kernel(const float4 *__restrict__ part, int npix4, int nx, int rpc, int n_bins, int tiles, int F,
+epi_reduce_frames_kernel(const float4 *part, int npix4, int nx, int rpc, int n_bins, int tiles, int F,
                          FrameDiv div, EpiOut out)
 {
     const int q = threadIdx.x >> 5, lane = threadIdx.x & 31, f = blockIdx.y * FR_N + q;
@@ -1106,9 +1106,8 @@ epi_reduce_frames_kernel(const float4 *__restrict__ part, int npix4, int nx, int
 // is not positive (a frame without a finite rho) gives rho_n = 0, the reading of
 // the padded maps; without it the division's result stands.
 __global__ void __launch_bounds__(EPI_THREADS)
-epi_normalize_kernel(const float4 *__restrict__ rho_tmp, const float4 *__restrict__ e_tmp,
-                     const unsigned *__restrict__ fmax, int npix4, bool guard, float4 *__restrict__ image,
-                     float4 *__restrict__ rho_n)
+epi_normalize_kernel(const float4 *rho_tmp, const float4 *e_tmp, const unsigned *fmax, int npix4, bool guard,
+                     float4 *__restrict__ image, float4 *__restrict__ rho_n)
 {
     const int f = blockIdx.y;
     const int x = blockIdx.x * EPI_THREADS + threadIdx.x;

@@ -81,7 +81,11 @@ __device__ __forceinline__ bool mbar_wait_sleep(uint64_t *bar, unsigned parity)
 // ---- programmatic dependent launch ----
 // Waits until the kernels this one depends on have completed and their writes
 // are visible (returns at once in a kernel launched without the attribute).
-// Every global read of their results and every global write comes after it.
+// Every global read of their results and every global write comes after it, and
+// those results are read through pointers that are not `const __restrict__`: that
+// promises data which nothing writes while the kernel is resident and allows
+// non-coherent loads, and here the kernel is resident while its predecessor writes.
+// Only tables that no kernel of a call writes keep the qualifier.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 // The next kernel of the stream may be scheduled from here on (its pdl_wait
 // still waits for this one's end). Called near a kernel's end, so that the
