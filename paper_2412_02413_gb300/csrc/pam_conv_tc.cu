@@ -120,18 +120,25 @@ __device__ float conv_chain(const uint4 *__restrict__ in, size_t plane, const ui
     return s;
 }
 
-// EXACT (training): the outputs are bit for bit those of the CUDA-core kernel,
-// so a gradient does not depend on which of the two computed the activations.
-// Both sum in FP32 and differ by the order only, which shows where a sum lies
-// within that difference of a BF16 rounding boundary or of the ReLU's zero:
+// EXACT (training): the outputs are, but for rare cases, those of the CUDA-core
+// kernel, so a gradient hardly depends on which of the two computed the
+// activations. Both sum in FP32 and differ by the order only, which shows where a
+// sum lies within that difference of a BF16 rounding boundary or of the ReLU's zero:
 // those outputs (about one in a thousand) are recomputed by conv_chain. An
 // epilogue warp collects them over its rows and recomputes 32 at a time, one
 // per lane: recomputing each row's few at once left most lanes idle (32 -> 32
 // layer, 16 frames of 512 x 128: 107 us forward and 185 us backward, against 59
-// and 78 us, with packed checks 53 and 66; 36 us without EXACT). The window is CHAIN_TOL times the pixel's largest sum: the chain of up to 288
-// roundings and the tensor core's 18 steps differ by about 1.5e-7 of it (one
-// standard deviation), a sixth of the window.
+// and 78 us, with packed checks 53 and 66; 36 us without EXACT).
+// The window on either side is CHAIN_TOL times the largest final sum of the
+// thread's 16 channels, and BIAS_TOL of the value itself for the rounding of the
+// bias addition. It is not a bound. The two orders (a chain of up to 288 roundings,
+// and the tensor core's 9 or 18 truncated steps) differ in proportion to the terms:
+// by 1.5e-7 of the largest sum (one standard deviation, a sixth of the window) for
+// trained and random weights, but by more of it where the terms cancel in all 16
+// channels at once. An output may then be the tensor core's rounding: within the same
+// n 2^-23 sum |x w| of the exact sum, n terms, before its rounding to BF16.
 constexpr float CHAIN_TOL = 9.5367431640625e-7f;   // 2^-20
+constexpr float BIAS_TOL = 2.384185791015625e-7f;  // 2^-22: two FP32 ulp at least
 
 template <int NCI, int NCO, int EPI, bool EXACT>
 __global__ void __launch_bounds__(threads(EXACT), EXACT ? 2 : 1)
@@ -338,7 +345,10 @@ conv_tc_kernel(const uint4 *__restrict__ in, const uint4 *__restrict__ wt, const
                     if constexpr (EPI == TC_RELU) v = __fadd2_rn(v, make_float2(b[2 * i], b[2 * i + 1]));
                     w[i] = EPI == TC_RELU ? pack2_relu(v.x, v.y) : pack2(v.x, v.y);
                     if constexpr (EXACT) {
-                        const float2 up = __fadd2_rn(v, make_float2(tol, tol)), dn = __fadd2_rn(v, make_float2(-tol, -tol));
+                        // an activation is positive, so the two ends move apart; an input gradient has no bias
+                        const float hi = EPI == TC_RELU ? 1.0f + BIAS_TOL : 1.0f, lo = EPI == TC_RELU ? 1.0f - BIAS_TOL : 1.0f;
+                        const float2 up = __ffma2_rn(v, make_float2(hi, hi), make_float2(tol, tol));
+                        const float2 dn = __ffma2_rn(v, make_float2(lo, lo), make_float2(-tol, -tol));
                         d[i] = EPI == TC_RELU ? pack2_relu(up.x, up.y) ^ pack2_relu(dn.x, dn.y)
                                               : pack2(up.x, up.y) ^ pack2(dn.x, dn.y);
                     }

@@ -39,12 +39,13 @@ namespace pam {
 cudaError_t launch_conv_tc(int layer, const uint4 *in, const uint4 *wt, const float *bias, void *out, int F, int H,
                            int *status, cudaStream_t st);
 cudaError_t prepare_conv_tc();
-// Hidden layers 0..3 for training: the same bits as the CUDA-core kernel's.
+// Hidden layers 0..3 for training: the CUDA-core kernel's values but for rare
+// roundings (pam_conv_tc.cu says which).
 cudaError_t launch_conv_tc_exact(int layer, const uint4 *in, const uint4 *wt, const float *bias, uint4 *out, int F,
                                  int H, int *status, cudaStream_t st);
 // tcgen05 input gradient of layer 1..4 through the ReLU of its input: the
 // convolution of dY with the adjoint weights, zero where `mask` (the layer's
-// input activation) is not positive; nx == 128 only, the CUDA-core kernel's bits.
+// input activation) is not positive; nx == 128 only, values as above.
 cudaError_t launch_conv_tc_grad(int layer, const uint4 *dY, const uint4 *wt, const uint4 *mask, uint4 *out, int F,
                                 int H, int *status, cudaStream_t st);
 // Weight gradients on the tensor cores (pam_wgrad.cu): wgrad_ctas partials of
@@ -802,9 +803,9 @@ cudaError_t run_forward(pam_learn_s *l, const uint4 *feat, int n, bool keep, cud
     }
     for (int k = 0; k < 4; ++k) {
         const uint4 *in = k ? a[k - 1] : feat;
-        // Without pam_learn_configure's tensor cores the activations are the
-        // CUDA-core kernel's bits; at nx = 128 tcgen05 makes the same bits faster
-        // (32 -> 32 layer, 16 frames of 512 x 128: 53 us against 467 us).
+        // Without pam_learn_configure's tensor cores the activations are FP32 sums in
+        // the CUDA-core kernel's order; at nx = 128 tcgen05 makes them, but for rare
+        // roundings, faster (32 -> 32 layer, 16 frames of 512 x 128: 53 us against 467 us).
         if (W == 128)
             e = pam::launch_conv_tc_exact(k, in, reinterpret_cast<const uint4 *>(l->prep.wtc[k]), l->prep.bias[k], a[k],
                                           n, H, l->plan->w.status, st);
