@@ -270,11 +270,9 @@ conv_tc_kernel(const uint4 *__restrict__ in, const uint4 *__restrict__ wt, const
             umma_commit_elect(&afull[t]);
             umma_commit_elect(&sfree[r % NSLOT]);
         }
-        if (!ok && any && lane == 0) {
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                             smem_u32(dbar))
-                         : "memory");
-            wait(dbar, 0);
+        if (any) {   // this warp's MMAs end before the tensor memory is freed, whichever warp gave up
+            umma_commit_elect(dbar);
+            mbar_wait(dbar, 0);
         }
         __syncwarp();
     } else {

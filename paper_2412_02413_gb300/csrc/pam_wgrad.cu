@@ -213,8 +213,8 @@ wgrad_tc_kernel(const uint4 *__restrict__ X, const uint4 *__restrict__ dY, int F
             ny += (unsigned)n;
             r += n;
         }
-        if (!ok && any && lane == 0) {
-            umma_commit(&dbar[v]);
+        if (any) {   // this warp's MMAs end before the tensor memory is freed, whichever warp gave up
+            umma_commit_elect(&dbar[v]);
             mbar_wait(&dbar[v], 0);
         }
         __syncwarp();
