@@ -164,7 +164,8 @@ def _stream_ptr(stream=None) -> int:
     if stream is not None:
         return int(stream.cuda_stream)
     torch = _require_cuda()
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)   # not a documented name
+    return int(torch.cuda.current_stream().cuda_stream) if raw is None else raw(torch.cuda.current_device())
 
 
 def _dptr(t) -> Optional[int]:
