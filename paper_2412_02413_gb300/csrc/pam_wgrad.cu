@@ -17,23 +17,28 @@
 // (frame after frame). Warp 0 stages each input row (three output rows use it)
 // and each dY row once, by bulk copies into two rings; warps 1-3 issue one column
 // shift's W / 16 MMAs (M = 128, N = 32 or 16, K = 16) per output row each; warps 4-7
-// add up db from the staged dY rows and, every FLUSH rows, add the accumulators of
+// add up db from the staged dY rows and, every SETK K steps, add the accumulators of
 // the three column shifts to FP32 sums in registers, while the MMAs go on into a
-// second set of accumulators (a chain of FLUSH W / 16 tensor-core steps keeps the
-// rounding of the accumulators, which the hardware truncates, below that of the
-// FP32 sums). The CTA writes one partial; wgrad_reduce_kernel adds the CTAs'
-// partials in order, so results do not depend on timing.
+// second set of accumulators. The hardware truncates the accumulators, a bias that
+// grows with the chain: over 8 steps (4 in the last layer, whose terms are often of
+// one sign and whose sums are one column to read) the error against 64-bit sums is
+// that of FP32 FMAs or less at every width, over 32 steps the last layer's was 2 to 7
+// times that (16 frames of 100 x 128, trained weights: 1.4e-7 of the gradient against
+// 1.15e-6, and 1.5e-7 with FMAs). The CTA writes one partial; wgrad_reduce_kernel adds
+// the CTAs' partials in order, so results do not depend on timing.
 //
 // A window of 16 groups of 8 channels is more than the three rows: the groups
 // past them read whatever the following slots hold, which only reaches
 // accumulator rows (or, with one dY chunk, columns) that nobody reads.
 //
-// Measured (GB300, 16 frames of 512 x 128): 47 us for 32 -> 32 channels, 42 us for
-// the first and last layers, where one issuing warp took 61 us, mma.sync 97 us (its
-// rate) and the CUDA cores 689 us. Bound by the hand-offs of a row (0.8 us):
-// halving the MMAs, dropping the db sums or deepening the rings changes it by less
-// than 5%, and DRAM runs at 3.1 TB/s. One MMA of N = 96 per 16 pixels, with dY
-// staged once per column shift, took 61 us (three times the copies).
+// Measured (GB300, 16 frames of 512 x 128): 49 us for 32 -> 32 channels, 45 us for
+// the first layer and 50 us for the last (47, 43 and 43 with chains of 32 steps),
+// where one issuing warp took 61 us, mma.sync 97 us (its rate) and the CUDA cores
+// 689 us. Bound by the hand-offs and the issue of a row (0.8 us): a branch beside each
+// MMA makes 61 us of it, while halving the MMAs, dropping the db sums, four
+// accumulator sets or deeper rings change it by less than 5%, and DRAM runs at
+// 3 TB/s. One MMA of N = 96 per 16 pixels, with dY staged once per column shift, took
+// 61 us (three times the copies).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -46,7 +51,6 @@ namespace {
 using namespace ptx;
 
 constexpr int NSX = 8, NSY = 6;    // ring slots of input rows and dY rows (NSY >= NSX - 2)
-constexpr int FLUSH = 4;           // output rows per accumulator set
 constexpr int THREADS = 256;
 constexpr int GROUPS = 16;         // 8-channel groups of M = 128
 
@@ -55,11 +59,15 @@ template <int NCI, int NCY>
 struct WG {
     static constexpr int NB = NCY == 1 ? 16 : 8 * NCY;     // GEMM columns (at least 16 for M = 128)
     static constexpr int VROWS = 3 * NCI * 8;              // accumulator rows in use
+    static constexpr int SETK = NCY == 1 ? 4 : 8;          // K steps (of 16 pixels) of an accumulator
+    static constexpr int HALVES = 8 / SETK;                // accumulators of a row of 128 pixels and column shift
     // input ring: NSX slots, the first two again behind the last (a window of
     // three rows is contiguous from any slot), and room for the rest of the window
     static constexpr int XSLOTS = NSX + 2;
     static constexpr int XCHUNKS = (NSX - 1) * NCI + GROUPS > XSLOTS * NCI ? (NSX - 1) * NCI + GROUPS : XSLOTS * NCI;
     static constexpr int YCHUNKS = NSY * NCY + 1;          // the second column group of NCY = 1 reads one further
+    static_assert(HALVES == 1 || NB == 16, "one accumulator per column shift where all columns are read");
+    static_assert(2 * 3 * HALVES * NB <= 256, "two accumulator sets in the tensor memory allocated");
     static constexpr size_t smem(int W) { return 1024 + (size_t)(XCHUNKS + YCHUNKS) * (W + 2) * 16; }
 };
 
@@ -125,6 +133,12 @@ wgrad_tc_kernel(const uint4 *__restrict__ X, const uint4 *__restrict__ dY, int F
         return true;
     };
 
+    // An accumulator set: SETK K steps in each accumulator, of 2^lrps rows or of half a row.
+    const int lrps = 16 * G::SETK > W ? 31 - __clz(16 * G::SETK / W) : 0;
+    const int halves = W > 16 * G::SETK ? G::HALVES : 1;
+    // Whether row `done` (of `rows`) of the share is the last of its set.
+    auto last_of_set = [lrps](int done, int rows) { return ((done + 1) & ((1 << lrps) - 1)) == 0 || done + 1 == rows; };
+
     // The share's rows, in segments of one frame: n output rows from row a of
     // frame f use n + 2 staged input rows (counted by nx) and n dY rows (ny).
     const long long T = (long long)F * H;
@@ -187,19 +201,29 @@ wgrad_tc_kernel(const uint4 *__restrict__ X, const uint4 *__restrict__ dY, int F
                     ok = wait(&xfull[(nx + i + k) % NSX], ((nx + i + k) / NSX) & 1u);
                 const unsigned y = ny + (unsigned)i;
                 if (ok) ok = wait(&yfull[y % NSY], (y / NSY) & 1u);
-                const int set = done / FLUSH, t = set & 1;
-                if (ok && done % FLUSH == 0 && set >= 2) ok = wait(&aempty[t], (unsigned)((set >> 1) - 1) & 1u);
+                const bool first = (done & ((1 << lrps) - 1)) == 0;
+                const int set = done >> lrps, t = set & 1;
+                if (ok && first && set >= 2) ok = wait(&aempty[t], (unsigned)((set >> 1) - 1) & 1u);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
                 const unsigned arow = xb + ((nx + (unsigned)i) % NSX) * (NCI * CHB) + (unsigned)v * 16u;
                 const unsigned brow = yb + (y % NSY) * (NCY * CHB) + 16u;   // dY has the border too
                 const uint64_t da0 = umma_desc(arow, 128, CHB), db0 = umma_desc(brow, 128, CHB);
-#pragma unroll 8
-                for (int ks = 0; ks < W / 16; ++ks)
-                    umma_elect(tmem + (unsigned)((t * 3 + v) * NB), da0 + (uint64_t)(ks * 16), db0 + (uint64_t)(ks * 16),
-                               idesc_mn(NB), (done % FLUSH || ks) ? 1u : 0u);
+                // K step k of the row, `per` steps to an accumulator
+                auto issue = [&](int k, int per) {
+                    umma_elect(tmem + (unsigned)(((t * 3 + v) * G::HALVES + k / per) * NB), da0 + (uint64_t)(k * 16),
+                               db0 + (uint64_t)(k * 16), idesc_mn(NB), (!first || k % per) ? 1u : 0u);
+                };
+                if (W == 128) {   // unrolled: issuing the MMAs is much of a row's time
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) issue(k, G::SETK);
+                } else {
+#pragma unroll 4
+                    for (int k = 0; k < W / 16; ++k) issue(k, 8);
+                }
                 any = true;
+                if (last_of_set(done, rows)) umma_commit_elect(&afull[t]);
                 umma_commit_elect(&xfree[(nx + i) % NSX]);
                 if (i == n - 1) {   // the segment's last two rows are not used again
                     umma_commit_elect(&xfree[(nx + i + 1) % NSX]);
@@ -207,7 +231,6 @@ wgrad_tc_kernel(const uint4 *__restrict__ X, const uint4 *__restrict__ dY, int F
                 }
                 umma_commit_elect(&yfree[y % NSY]);
                 ++done;
-                if (done % FLUSH == 0 || done == rows) umma_commit_elect(&afull[t]);
             }
             nx += (unsigned)n + 2u;
             ny += (unsigned)n;
@@ -245,25 +268,28 @@ wgrad_tc_kernel(const uint4 *__restrict__ X, const uint4 *__restrict__ dY, int F
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&yfree[y % NSY]);
-            if ((y + 1) % FLUSH != 0 && y + 1 != rows) continue;
-            const int set = y / FLUSH, t = set & 1;
+            if (!last_of_set(y, rows)) continue;
+            const int set = y >> lrps, t = set & 1;
             if (!__all_sync(0xffffffffu, wait(&afull[t], (unsigned)(set >> 1) & 1u))) break;
             tc_fence_after();
-            const unsigned ta = tmem + (unsigned)(t * 3 * NB) + ((unsigned)(32 * quarter) << 16);
+            const unsigned ta = tmem + (unsigned)(t * 3 * G::HALVES * NB) + ((unsigned)(32 * quarter) << 16);
+            if constexpr (NB == 32) {
 #pragma unroll
-            for (int v = 0; v < 3; ++v) {
-                if constexpr (NB == 32) {
+                for (int v = 0; v < 3; ++v) {
                     unsigned q[32];
                     tmem_ld32(ta + (unsigned)(v * NB), q);
                     tmem_wait_ld();
 #pragma unroll
                     for (int o = 0; o < 32; ++o) sum[v][o] += __uint_as_float(q[o]);
-                } else {
-                    float q[4];
-                    tmem_ld4(ta + (unsigned)(v * NB), q);
-                    tmem_wait_ld();
-                    sum[v][0] += q[0];
                 }
+            } else {
+                float q[3 * G::HALVES][4];
+#pragma unroll
+                for (int a = 0; a < 3 * G::HALVES; ++a) tmem_ld4(ta + (unsigned)(a * NB), q[a]);
+                tmem_wait_ld();
+#pragma unroll
+                for (int a = 0; a < 3 * G::HALVES; ++a)
+                    if (a % G::HALVES < halves) sum[a / G::HALVES][0] += q[a][0];
             }
             tc_fence_before();
             __syncwarp();

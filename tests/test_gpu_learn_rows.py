@@ -82,3 +82,46 @@ def test_gradients_of_many_rows(ne, nz, frames, parts):
             err = np.abs(got[li][k] - want[li][k])
             m = m + 1e-5 * m.max()
             assert np.all(err <= tol * m), (li, k, float(np.max(err / m)), tol)
+
+
+def bf16(x):
+    return x.float().bfloat16().double()
+
+
+def chain(x, w):
+    """s = fma(x, w, s) in FP32 over input channels, then taps."""
+    xs = shifted(x)
+    s = torch.zeros((x.shape[0], w.shape[0]) + x.shape[2:], dtype=torch.float64, device="cuda")
+    for c in range(x.shape[1]):
+        for t in range(9):
+            s = (xs[t][:, None, c] * w[None, :, c, t // 3, t % 3, None, None] + s).float().double()
+    return s
+
+
+@pytest.mark.parametrize("ne,nz,frames", [(128, 100, 16), (64, 256, 4)])
+def test_last_layers_weight_sums_round_without_bias(ne, nz, frames):
+    """With targets below every prediction dL/dz is positive, as the last layer's input is: its weight gradients are
+    sums of terms of one sign, where truncated additions add up. 64-bit sums of the same BF16 operands."""
+    L, _ = _learned(ne, 128, nz, max_frames=frames)
+    params = rand_params(45)
+    L.set_params(flat(params))
+    x, feats = _features(frames, nz, ne, 46)
+    g, _ = L.grads(feats, torch.zeros((frames, nz, ne), device="cuda"))
+    L.sync()
+    got = unflat(g.cpu().numpy().astype(np.float64))[4][0]
+    L.close()
+    h = xt = torch.from_numpy(x).cuda()
+    for li, (w, b) in enumerate(gpu_weights(params)):
+        z = (chain(h, torch.from_numpy(w).cuda()) + torch.from_numpy(b).cuda()[None, :, None, None]).float().double()
+        if li < 4:
+            h = bf16(z.clamp_min(0.0))
+    s = torch.sigmoid(z)
+    wgt = 0.05 + 0.95 * (10.0 ** (4 * xt[:, :1]) - 1e-4).clamp(0, 1)
+    dy = bf16(2.0 * wgt * (EPS + (1 - EPS) * s) / s.numel() * (1 - EPS) * s * (1 - s))
+    o = dy.transpose(0, 1).reshape(1, -1)
+    want = torch.stack([o @ v.transpose(0, 1).reshape(32, -1).T for v in shifted(h)], -1).cpu().numpy()
+    err = np.linalg.norm(got.reshape(want.shape) - want) / np.linalg.norm(want)
+    # A truncated step loses half an ulp, 2^-24, of a partial sum that is half its final size on average: four steps
+    # 1.2e-7 (sets of 64 pixels) and eight 2.4e-7; unbiased FP32 rounding of the 152 shares and the values of dL/dz
+    # that expf's last bits turn (one in 2^12 by 2^-9) add 1e-7
+    assert err <= 4e-7, err
