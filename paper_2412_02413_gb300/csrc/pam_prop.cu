@@ -1613,9 +1613,9 @@ cudaError_t launch_epilogue(const pam_plan_s &p, int n_frames, int napq, int n_s
 // Measured (GB300, whole calls, us, unsplit / this split): nx = 128, 9 items 1058 / 141
 // with 300 bins, 77 / 51 with 10; nx = 32, 4 items 128 / 48 with 40. Against the best of
 // splits 1 to 48 over widths 16 to 128, 1 to 180 items and 3 to 300 bins it is 1.3 %
-// slower on average and never more than the timer's step slower than unsplit, where a
-// rule without bins and width (48 chunks for one item) took 130 for 107 us (nx = 64,
-// 100 items of 5 bins). The gate tiles of 32 frames (32 items of 32 rows x 300 bins at
+// slower on average and never more than the timer's step slower than unsplit; a rule
+// without bins and width (48 chunks for one item) took 130 us where this one takes 89
+// (nx = 64, 100 items of 5 bins). The gate tiles of 32 frames (32 items of 32 rows x 300 bins at
 // nx = 128) take 175 us and 26 us for the sums, against 705 us unsplit.
 constexpr int kMaxItemSplit = 48, kMaxItemUnits = 1024;
 int item_split(int nx, int napq, int rpl, int n_items, int n_bins, int sms, size_t floats)
